@@ -1144,9 +1144,21 @@ void launch_dslash_epi_t(const eofa_ctx* ctx, int par, const void* in, void* out
     EOFA_LAUNCHED();
 }
 
+template <int P>
+bool try_pair(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, cudaStream_t st) {
+    if constexpr (P == P32) return pair_dslash_p32(ctx, par, dag, a, st);
+    else if constexpr (P == P16) return pair_dslash_p16(ctx, par, dag, a, st);
+    else return false;
+}
+
 template <int P, int MODE>
 void dslash_epi_prec(const eofa_ctx* ctx, int par, int dag, const void* in, void* out, const Op5& op, const void* y,
                      double a_out, double b_in, double* red, int slot, const Epi& ep, cudaStream_t st) {
+    if (try_pair<P>(ctx, par, dag,
+                    PairArgs{MODE, in, out, MODE == 2 ? nullptr : &op, y, a_out, b_in, red, slot,
+                             MODE == 1 ? &ep.op2 : nullptr, ep.out2, ep.aux, ep.out3, ep.aux2, ep.it, ep.slot2},
+                    st))
+        return;
 #define EPI_CASE(L)                                                                                      \
     if (dag) launch_dslash_epi_t<P, 1, L, MODE>(ctx, par, in, out, op, y, a_out, b_in, red, slot, ep, st); \
     else launch_dslash_epi_t<P, 0, L, MODE>(ctx, par, in, out, op, y, a_out, b_in, red, slot, ep, st);
@@ -1180,6 +1192,8 @@ void launch_local5_t(const eofa_ctx* ctx, const Op5& op, const void* x, const vo
 template <int P>
 void dslash_prec(const eofa_ctx* ctx, int par, int dag, const void* in, void* out, const Op5& op, const void* y,
                  double a_out, double b_in, double* red, int slot, cudaStream_t st) {
+    const bool hasop = op.inv[0] || op.inv[1] || op.fwd[0] || op.fwd[1] || op.sigma[0] != 0.0 || op.sigma[1] != 0.0;
+    if (try_pair<P>(ctx, par, dag, PairArgs{0, in, out, hasop ? &op : nullptr, y, a_out, b_in, red, slot}, st)) return;
 #define DSL_CASE(L)                                                                             \
     if (dag) launch_dslash_t<P, 1, L>(ctx, par, in, out, op, y, a_out, b_in, red, slot, st);   \
     else launch_dslash_t<P, 0, L>(ctx, par, in, out, op, y, a_out, b_in, red, slot, st);

@@ -52,5 +52,28 @@ void fused_xp_update(const eofa_ctx* ctx, int prec, int precx, const double* sc,
                      const void* s, cudaStream_t st);
 Op5 op_identity();
 
+// The two-slices-per-thread kernels (dslash_pair.cuh).  mode and the fields
+// behind it are the MODEs of dslash_impl.cuh; op null: B = 1.  The blocks are
+// finalized (op_finalize).  False, with nothing launched, when the launch is
+// not one they take.
+struct PairArgs {
+    int mode;
+    const void* in;
+    void* out;
+    const Op5* op;
+    const void* y;
+    double a_out, b_in;
+    double* red;
+    int slot;
+    const Op5* op2 = nullptr;
+    void* out2 = nullptr;
+    const void* aux = nullptr;
+    void* out3 = nullptr;
+    const void* aux2 = nullptr;
+    int it = 0, slot2 = 0;
+};
+bool pair_dslash_p32(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, cudaStream_t st);
+bool pair_dslash_p16(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, cudaStream_t st);
+
 // throws EOFA_ETIMEOUT (and clears the word) when a kernel's bounded wait ran out
 void check_device_error(const eofa_ctx* ctx, cudaStream_t st);
