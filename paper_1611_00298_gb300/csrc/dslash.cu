@@ -33,13 +33,13 @@ void fused_dslash(const eofa_ctx* ctx, int prec, int out_parity, int dagger, con
 
 void fused_local5(const eofa_ctx* ctx, int prec, const Op5& op, const void* x, const void* z, double c0,
                   const double* sc, int it, int use_alpha, void* xw, void* out, double a_out, double* red, int slot,
-                  cudaStream_t st) {
+                  cudaStream_t st, const void* y, double b_in) {
     const Op5 opf = op_finalize(op, ctx->Ls);
-    const double nf = 1.0 + (z ? 1.0 : 0.0) + (xw ? 1.0 : 0.0) + (out ? 1.0 : 0.0);
+    const double nf = 1.0 + (z ? 1.0 : 0.0) + (xw ? 1.0 : 0.0) + (out ? 1.0 : 0.0) + (y ? 1.0 : 0.0);
     prof_begin(ctx, 3 + prec, st, (double)ctx->Vh * ctx->Ls * spinor_bytes(prec) * nf);
-    if (prec == P64) local5_p64(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st);
-    else if (prec == P32) local5_p32(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st);
-    else local5_p16(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st);
+    if (prec == P64) local5_p64(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st);
+    else if (prec == P32) local5_p32(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st);
+    else local5_p16(ctx, opf, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st);
     prof_end(ctx, st);
 }
 

@@ -156,17 +156,46 @@ __device__ __forceinline__ void project(const cpx<R>* psi, cpx<R>* h) {
     }
 }
 
-template <int MU, int SG, typename R>
+__device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
+
+// u . h (three complex products) as two chains of multiply-adds, 12
+// instructions instead of the 16 of three products and two sums: the FP64
+// hop runs at the FP64 pipe's rate (1056 instructions a site and slice at
+// 24^3 x 64 x 24 in 20.9 ms), so its time is the instruction count.
+template <typename R>
+__device__ __forceinline__ cpx<R> row_dot(const cpx<R>* u, const cpx<R>* h) {
+    R re = u[0].re * h[0].re, im = u[0].re * h[0].im;
+    re = fma_r(-u[0].im, h[0].im, re);
+    im = fma_r(u[0].im, h[0].re, im);
+#pragma unroll
+    for (int k = 1; k < 3; k++) {
+        re = fma_r(u[k].re, h[k].re, re);
+        im = fma_r(u[k].re, h[k].im, im);
+        re = fma_r(-u[k].im, h[k].im, re);
+        im = fma_r(u[k].im, h[k].re, im);
+    }
+    return mk(re, im);
+}
+
+// FIRST: the accumulators are still zero and take the row instead of adding it
+template <int MU, int SG, bool FIRST = false, typename R>
 __device__ __forceinline__ void mac_row(const cpx<R>* u, int a, const cpx<R>* h, cpx<R>* acc) {
-    const cpx<R> w0 = cmul(u[0], h[0]) + cmul(u[1], h[1]) + cmul(u[2], h[2]);
-    const cpx<R> w1 = cmul(u[0], h[3]) + cmul(u[1], h[4]) + cmul(u[2], h[5]);
-    acc[a] = acc[a] + w0;
-    acc[3 + a] = acc[3 + a] + w1;
+    const cpx<R> w0 = row_dot(u, h), w1 = row_dot(u, h + 3);
     cpx<R> l0, l1;
     if (MU == 0) { l0 = itimes(w1); l1 = itimes(w0); }
     else if (MU == 1) { l0 = w1; l1 = mk(-w0.re, -w0.im); }
     else if (MU == 2) { l0 = itimes(w0); l1 = mitimes(w1); }
     else { l0 = w0; l1 = w1; }
+    if (FIRST) {
+        acc[a] = w0;
+        acc[3 + a] = w1;
+        acc[6 + a] = SG > 0 ? l0 : mk(-l0.re, -l0.im);
+        acc[9 + a] = SG > 0 ? l1 : mk(-l1.re, -l1.im);
+        return;
+    }
+    acc[a] = acc[a] + w0;
+    acc[3 + a] = acc[3 + a] + w1;
     acc[6 + a] = SG > 0 ? acc[6 + a] + l0 : acc[6 + a] - l0;
     acc[9 + a] = SG > 0 ? acc[9 + a] + l1 : acc[9 + a] - l1;
 }
@@ -208,7 +237,7 @@ __device__ __forceinline__ void hop_mu(const Geom& g, int par, int j, const int*
             link_row<R>(gauge, lidx, a, dirn == 1, u);
 #pragma unroll
             for (int k = 0; k < SPT; k++) {
-                if (dirn == 0) mac_row<MU, DAG ? 1 : -1>(u, a, h[k], acc[k]);
+                if (dirn == 0) mac_row<MU, DAG ? 1 : -1, MU == 0>(u, a, h[k], acc[k]);
                 else mac_row<MU, DAG ? -1 : 1>(u, a, h[k], acc[k]);
             }
         }
@@ -422,9 +451,64 @@ __device__ __forceinline__ void col_stream_f2(const Half<float>& H, cpx<float>* 
     }
 }
 
-// apply B to the column at col (shared memory, stride 1, length Ls)
+template <typename R>
+__device__ __forceinline__ cpx<R> fma_cr(R a, cpx<R> x, cpx<R> y) {
+    return mk(fma_r(a, x.re, y.re), fma_r(a, x.im, y.im));
+}
+
+// Whether the columns of op run as col_lead: FP64 (bound by the FP64 pipe) and
+// every Ls without an unrolled build; op_finalize says whether op has the form.
 template <typename R, int LS>
+__device__ __forceinline__ bool has_lead(const Op5& op) {
+    return (LS == 0 || std::is_same<R, double>::value) && op.lead[0] != 0.0 && op.lead[1] != 0.0;
+}
+
+// B without its leading factor: with v = p1 u the inverse is v_s = x_s + mr v_{s-1}
+// and B x / lead = v_s + (q2 / p2) v_{s-1}, v_{-1} = -mass v_{Ls-1}: three
+// multiply-adds per real component (the Horner sum of the corner, the
+// recurrence, the matrix) instead of the five of col_stream; the caller's
+// scale carries lead.
+template <typename R, int LS, bool R1>
+__device__ __forceinline__ void col_lead(const Op5& op, int h, int Lsr, cpx<R>* col, const R* wv) {
+    const int Ls = LS > 0 ? LS : Lsr;
+    const R mass = (R)op.mass, mr = (R)(h ? op.mr[1] : op.mr[0]), nrm = (R)(h ? op.nrm[1] : op.nrm[0]);
+    const R rat = (R)(h ? op.ratio[1] : op.ratio[0]);
+    const R *w = wv + 2 * h * Ls, *vv = wv + (2 * h + 1) * Ls;
+    const bool up = (h ? op.dir1[1] : op.dir1[0]) == 0;
+    cpx<R>* c0 = up ? col : col + (Ls - 1);
+    const R* v0 = up ? vv : vv + (Ls - 1);
+    const int st = up ? 1 : -1;
+    cpx<R> acc = mk(R(0), R(0)), d = mk(R(0), R(0));
+#pragma unroll
+    for (int s = 1; s < Ls; s++) acc = fma_cr(mr, acc, lds(c0 + s * st));
+    const cpx<R> first = nrm * fma_cr(-mass * mr, acc, lds(c0));
+    cpx<R> v = first;
+    if (R1) d = v0[0] * first;
+#pragma unroll
+    for (int s = 1; s < Ls; s++) {
+        const cpx<R> vn = fma_cr(mr, v, lds(c0 + s * st));
+        if (R1) d = fma_cr(v0[s * st], vn, d);
+        sts(c0 + s * st, fma_cr(rat, v, vn));
+        v = vn;
+    }
+    sts(c0, fma_cr(-rat * mass, v, first));
+    if (R1) {
+        const cpx<R> sd = (R)(h ? op.sigl[1] : op.sigl[0]) * d;
+#pragma unroll
+        for (int s = 0; s < Ls; s++) sts(col + s, fma_cr(w[s], sd, lds(col + s)));
+    }
+}
+
+// apply B to the column at col (shared memory, stride 1, length Ls); LEAD: the
+// caller multiplies by op.lead when has_lead
+template <typename R, int LS, bool LEAD = false>
 __device__ __forceinline__ void column_op(const Op5& op, int c, cpx<R>* col, int Ls, const R* wv) {
+    if (LEAD && has_lead<R, LS>(op)) {
+        const int h = c < 6 ? 0 : 1;
+        if ((h ? op.sigma[1] : op.sigma[0]) == 0.0) col_lead<R, LS, false>(op, h, Ls, col, wv);
+        else col_lead<R, LS, true>(op, h, Ls, col, wv);
+        return;
+    }
     const Half<R> H = half_of<R>(op, c < 6 ? 0 : 1, wv, Ls);
     if (LS > 0 && H.inv && (!H.fwd || H.dir2 == H.dir1)) {
         if constexpr (EOFA_PACKED_F32 && std::is_same<R, float>::value) {
@@ -448,9 +532,10 @@ __device__ __forceinline__ void column_op(const Op5& op, int c, cpx<R>* col, int
 }
 
 // the column phase of a tile: one thread per (site, component) column
-template <typename R, int LS>
+template <typename R, int LS, bool LEAD = false>
 __device__ __forceinline__ void columns(const Op5& op, cpx<R>* sm, int ncols, int LsP, int Ls, const R* wv) {
-    for (int idx = threadIdx.x; idx < ncols; idx += blockDim.x) column_op<R, LS>(op, idx % 12, sm + idx * LsP, Ls, wv);
+    for (int idx = threadIdx.x; idx < ncols; idx += blockDim.x)
+        column_op<R, LS, LEAD>(op, idx % 12, sm + idx * LsP, Ls, wv);
 }
 
 __device__ __forceinline__ bool op_is_identity(const Op5& op) {
@@ -631,16 +716,14 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
     for (int k = 0; k < SPT; k++) sv[k] = sh + k * Lt;
     const bool active_thread = ls < NS;
     const int ntiles = (g.Vh + NS - 1) / NS;
-    const R scale = (R)(-0.5 * a_out);
+    // (the columns leave out / lead where the block has a leading factor)
+    const bool lead = HASOP && has_lead<R, LS>(op);
+    const R scale = (R)(-0.5 * a_out * (lead ? op.lead[0] : 1.0)), scale1 = (R)(-0.5 * a_out * (lead ? op.lead[1] : 1.0));
     double nacc = 0.0, nacc2 = 0.0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int j = tile * NS + ls;
         const bool site_ok = active_thread && j < g.Vh;
         cpx<R> acc[SPT][12];
-#pragma unroll
-        for (int k = 0; k < SPT; k++)
-#pragma unroll
-            for (int c = 0; c < 12; c++) acc[k][c] = mk(R(0), R(0));
         if (site_ok) {
             // the eight neighbour entries are loaded up front, so that no
             // spinor load waits behind the load of its own index
@@ -664,7 +747,7 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
             }
             __syncthreads();
             const int nsites = min(NS, g.Vh - tile * NS);
-            columns<R, LS>(op, sm, nsites * 12, LsP, Ls, wv_s);
+            columns<R, LS, true>(op, sm, nsites * 12, LsP, Ls, wv_s);
             __syncthreads();
             if (site_ok) {
 #pragma unroll
@@ -676,15 +759,22 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
         if (site_ok) {
 #pragma unroll
             for (int k = 0; k < SPT; k++) {
+                if (y == nullptr) {
 #pragma unroll
-                for (int c = 0; c < 12; c++) acc[k][c] = scale * acc[k][c];
-                if (y != nullptr) {
+                    for (int c = 0; c < 12; c++) acc[k][c] = (c < 6 ? scale : scale1) * acc[k][c];
+                } else {
                     cpx<R> yv[12];
                     if (EOFA_STREAM_HINTS) Field<P>::load_stream(y, j, sv[k], Ls, n5, yv);
                     else Field<P>::load(y, j, sv[k], Ls, n5, yv);
-                    const R bb = (R)b_in;
+                    if (b_in == 1.0) {
 #pragma unroll
-                    for (int c = 0; c < 12; c++) acc[k][c] = acc[k][c] + bb * yv[c];
+                        for (int c = 0; c < 12; c++) acc[k][c] = fma_cr(c < 6 ? scale : scale1, acc[k][c], yv[c]);
+                    } else {
+                        const R bb = (R)b_in;
+#pragma unroll
+                        for (int c = 0; c < 12; c++)
+                            acc[k][c] = fma_cr(c < 6 ? scale : scale1, acc[k][c], bb * yv[c]);
+                    }
                     if (MODE == 2 && ep.out2 != nullptr) {
                         // r <- r - alpha y
                         cpx<R> rv[12];
@@ -737,11 +827,16 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
             }
             __syncthreads();
             const int nsites = min(NS, g.Vh - tile * NS);
-            columns<R, LS>(ep.op2, sm, nsites * 12, LsP, Ls, wv2_s);
+            columns<R, LS, true>(ep.op2, sm, nsites * 12, LsP, Ls, wv2_s);
             __syncthreads();
             if (site_ok) {
 #pragma unroll
                 for (int c = 0; c < 12; c++) acc[0][c] = lds(sm + (ls * 12 + c) * LsP + sv[0]);
+                if (has_lead<R, LS>(ep.op2)) {
+                    const R f0 = (R)ep.op2.lead[0], f1 = (R)ep.op2.lead[1];
+#pragma unroll
+                    for (int c = 0; c < 12; c++) acc[0][c] = (c < 6 ? f0 : f1) * acc[0][c];
+                }
                 Field<P>::store_stream(ep.out2, j, sv[0], Ls, n5, acc[0]);
             }
         }
@@ -756,7 +851,8 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
 }
 
 // x' = x + c z (c = -alpha from the device scalars when use_alpha, else c0);
-// xw <- x' (if xw), |x'|^2 -> red[slot] (if red), out = a B x' (if out).
+// xw <- x' (if xw), |x'|^2 -> red[slot] (if red), out = a B x' + b y (if out; y may be null
+// and may be out).
 #ifndef EOFA_LOCAL5_MINB
 #define EOFA_LOCAL5_MINB 2
 #endif
@@ -765,7 +861,8 @@ __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MI
 template <int P, int LS>
 __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, Op5 op, const void* x, const void* z, double c0,
                                                      const double* sc, int it, int use_alpha, void* xw, void* out,
-                                                     double a_out, double* red, int slot, int NS) {
+                                                     double a_out, const void* y, double b_in, double* red, int slot,
+                                                     int NS) {
     typedef typename Field<P>::R R;
     extern __shared__ __align__(128) unsigned char smraw[];
     cpx<R>* sm = reinterpret_cast<cpx<R>*>(smraw);
@@ -777,6 +874,8 @@ __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, O
     const bool ident = op_is_identity(op);
     const int ntiles = (g.Vh + NS - 1) / NS;
     const R c = (R)(use_alpha ? -cg_alpha(sc, it) : c0);
+    const bool lead = has_lead<R, LS>(op);
+    const R f0 = (R)(a_out * (lead ? op.lead[0] : 1.0)), f1 = (R)(a_out * (lead ? op.lead[1] : 1.0));
     __shared__ R wv_s[4 * EOFA_MAX_LS];
     if (out && !ident) {
         stage_wv<R>(op, Ls, wv_s);
@@ -811,8 +910,7 @@ __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, O
                 }
                 __syncthreads();
                 const int nsites = min(NS, g.Vh - tile * NS);
-                for (int idx = threadIdx.x; idx < nsites * 12; idx += blockDim.x)
-                    column_op<R, LS>(op, idx % 12, sm + idx * LsP, Ls, wv_s);
+                columns<R, LS, true>(op, sm, nsites * 12, LsP, Ls, wv_s);
                 __syncthreads();
                 if (site_ok) {
 #pragma unroll
@@ -820,8 +918,16 @@ __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, O
                 }
             }
             if (site_ok) {
+                if (y == nullptr) {
 #pragma unroll
-                for (int k = 0; k < 12; k++) v[k] = (R)a_out * v[k];
+                    for (int k = 0; k < 12; k++) v[k] = (k < 6 ? f0 : f1) * v[k];
+                } else {
+                    cpx<R> yv[12];
+                    Field<P>::load_stream(y, j, s, Ls, n5, yv);
+                    const R bb = (R)b_in;
+#pragma unroll
+                    for (int k = 0; k < 12; k++) v[k] = fma_cr(k < 6 ? f0 : f1, v[k], bb * yv[k]);
+                }
                 if (EOFA_STREAM_HINTS) Field<P>::store_stream(out, j, s, Ls, n5, v);
                 else Field<P>::store(out, j, s, Ls, n5, v);
             }
@@ -1174,7 +1280,8 @@ void dslash_epi_prec(const eofa_ctx* ctx, int par, int dag, const void* in, void
 
 template <int P, int LS>
 void launch_local5_t(const eofa_ctx* ctx, const Op5& op, const void* x, const void* z, double c0, const double* sc,
-                     int it, int use_alpha, void* xw, void* out, double a_out, double* red, int slot, cudaStream_t st) {
+                     int it, int use_alpha, void* xw, void* out, double a_out, const void* y, double b_in, double* red,
+                     int slot, cudaStream_t st) {
     typedef typename Field<P>::R R;
     Geom g = ctx_geom(ctx);
     const int NS = pick_ns(g.Ls, sizeof(cpx<R>));
@@ -1184,7 +1291,7 @@ void launch_local5_t(const eofa_ctx* ctx, const Op5& op, const void* x, const vo
     auto k = local5_kernel<P, LS>;
     if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     unsigned grid = grid_size(k, threads, smem, ntiles, ctx->sms);
-    k<<<grid, threads, smem, st>>>(g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, NS);
+    k<<<grid, threads, smem, st>>>(g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, NS);
     EOFA_LAUNCHED();
 }
 
@@ -1209,13 +1316,14 @@ void dslash_prec(const eofa_ctx* ctx, int par, int dag, const void* in, void* ou
 
 template <int P>
 void local5_prec(const eofa_ctx* ctx, const Op5& op, const void* x, const void* z, double c0, const double* sc,
-                 int it, int use_alpha, void* xw, void* out, double a_out, double* red, int slot, cudaStream_t st) {
+                 int it, int use_alpha, void* xw, void* out, double a_out, const void* y, double b_in, double* red,
+                     int slot, cudaStream_t st) {
     switch (ctx->Ls) {
-        case 8: launch_local5_t<P, 8>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st); break;
-        case 12: launch_local5_t<P, 12>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st); break;
-        case 16: launch_local5_t<P, 16>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st); break;
-        case 24: launch_local5_t<P, 24>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st); break;
-        default: launch_local5_t<P, 0>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st); break;
+        case 8: launch_local5_t<P, 8>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st); break;
+        case 12: launch_local5_t<P, 12>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st); break;
+        case 16: launch_local5_t<P, 16>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st); break;
+        case 24: launch_local5_t<P, 24>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st); break;
+        default: launch_local5_t<P, 0>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st); break;
     }
 }
 
@@ -1238,8 +1346,8 @@ void xp_update_prec(const eofa_ctx* ctx, const double* sc, int it, void* x, void
     void dslash_##NAME(const eofa_ctx* ctx, int par, int dag, const void* in, void* out, const Op5& op,         \
                        const void* y, double a_out, double b_in, double* red, int slot, cudaStream_t st);       \
     void local5_##NAME(const eofa_ctx* ctx, const Op5& op, const void* x, const void* z, double c0,            \
-                       const double* sc, int it, int use_alpha, void* xw, void* out, double a_out, double* red, \
-                       int slot, cudaStream_t st);                                                              \
+                       const double* sc, int it, int use_alpha, void* xw, void* out, double a_out,              \
+                       const void* y, double b_in, double* red, int slot, cudaStream_t st);                                                              \
     void xp_update_##NAME(const eofa_ctx* ctx, const double* sc, int it, void* x, void* p, const void* s,      \
                           cudaStream_t st);                                                                     \
     void dslash_to_##NAME(const eofa_ctx* ctx, int par, int dag, const void* in, void* out, const Op5& op,      \
@@ -1261,9 +1369,9 @@ DSL_DECLARE(p16)
         dsl::dslash_prec<P>(ctx, par, dag, in, out, op, y, a_out, b_in, red, slot, st);                        \
     }                                                                                                           \
     void local5_##NAME(const eofa_ctx* ctx, const Op5& op, const void* x, const void* z, double c0,            \
-                       const double* sc, int it, int use_alpha, void* xw, void* out, double a_out, double* red, \
-                       int slot, cudaStream_t st) {                                                             \
-        dsl::local5_prec<P>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, red, slot, st);               \
+                       const double* sc, int it, int use_alpha, void* xw, void* out, double a_out,              \
+                       const void* y, double b_in, double* red, int slot, cudaStream_t st) {                                                             \
+        dsl::local5_prec<P>(ctx, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, st);      \
     }                                                                                                           \
     void xp_update_##NAME(const eofa_ctx* ctx, const double* sc, int it, void* x, void* p, const void* s,      \
                           cudaStream_t st) {                                                                    \

@@ -43,10 +43,11 @@ void fused_dslash_z(const eofa_ctx* ctx, int prec, int out_parity, int dagger, c
 void fused_dslash_x(const eofa_ctx* ctx, int prec, int out_parity, int dagger, const void* in, void* out,
                     const Op5& op, double* red, int it, void* x, const void* p, void* r, const void* q, int rslot,
                     cudaStream_t st);
-// x' = x + c z (c = -alpha(sc, it) if use_alpha else c0); xw <- x'; |x'|^2 -> red[slot]; out = a_out B x'
+// x' = x + c z (c = -alpha(sc, it) if use_alpha else c0); xw <- x'; |x'|^2 -> red[slot];
+// out = a_out B x' + b_in y
 void fused_local5(const eofa_ctx* ctx, int prec, const Op5& op, const void* x, const void* z, double c0,
                   const double* sc, int it, int use_alpha, void* xw, void* out, double a_out, double* red, int slot,
-                  cudaStream_t st);
+                  cudaStream_t st, const void* y = nullptr, double b_in = 0.0);
 // x += alpha p (skipped when x is null); p = s + beta p   (alpha, beta from sc at iteration it)
 void fused_xp_update(const eofa_ctx* ctx, int prec, int precx, const double* sc, int it, void* x, void* p,
                      const void* s, cudaStream_t st);

@@ -89,6 +89,10 @@ struct Op5 {
     // derived constants of the inverse (filled by op_finalize on the host):
     // mr = -q1/p1, invp = 1/p1, invN = 1/(p1 (1 + mass mr^Ls))
     double mr[2], invp[2], invN[2];
+    // the same block without its leading factor (col_lead, dslash_impl.cuh): lead = p2 / p1 (1 / p1
+    // without a matrix), ratio = q2 / p2, nrm = 1 / (1 + mass mr^Ls), sigl = sigma / p2; lead 0:
+    // no inverse, p2 = 0 or two directions
+    double lead[2], ratio[2], nrm[2], sigl[2];
 };
 Op5 op_finalize(Op5 op, int Ls);
 

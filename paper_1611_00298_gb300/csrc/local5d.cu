@@ -12,124 +12,91 @@
 // their transposes, and the EOFA rank-one corrections by Sherman-Morrison)
 // a product of at most one such inverse and one such matrix.
 //
-// A block of threads stages NS whole 4D sites (12 x Ls complex each) in
-// shared memory with coalesced loads, one thread per (site, component) runs
-// the recurrences over s, and the result is written back per (site, s).
+// Blocks without an inverse (D-tilde, M) are a two-point stencil in s: one
+// thread per (site, s) reads its slice and, through L1, the neighbouring one
+// of each chirality.  All others run as the launch of the CG's residual update
+// without its update (local5_kernel, dslash_impl.cuh): whole 4D sites staged in
+// shared memory, one thread per (site, component) column.
+//
+// What bounds them: the generic column loops that both kinds ran as before
+// reached 0.62 TB/s in FP64 (serial shared-memory steps).  The stencil takes
+// 48 to 72 FP64 instructions a site and slice, the columns 3 per real number.
+// D_DWF and D_DWF^+ on a 16^3 x 32 x 12 field (8 such passes and 4 hops):
+// 9.05 -> 6.74 ms with the hop's own share (4 x 1.61 -> 4 x 1.25 ms).
 #include "field.cuh"
+#include "fused.h"
 
 namespace {
 
-template <typename R>
-__device__ void inv_bidiag(cpx<R>* x, int Ls, R p, R q, int dir, R mass) {
-    R r = q / p;
-    R mr = -r;
-    R pw = 1;
-    for (int k = 0; k < Ls; k++) pw *= mr;
-    R N = p * (R(1) + mass * pw);
-    cpx<R> acc = mk(R(0), R(0));
-    if (dir == 0) {
-        for (int s = 1; s < Ls; s++) acc = mr * acc + x[s];
-        acc = mr * acc;
-        x[0] = (R(1) / N) * (x[0] - mass * acc);
-        for (int s = 1; s < Ls; s++) x[s] = (R(1) / p) * (x[s] - q * x[s - 1]);
-    } else {
-        for (int s = Ls - 2; s >= 0; s--) acc = mr * acc + x[s];
-        acc = mr * acc;
-        x[Ls - 1] = (R(1) / N) * (x[Ls - 1] - mass * acc);
-        for (int s = Ls - 2; s >= 0; s--) x[s] = (R(1) / p) * (x[s] - q * x[s + 1]);
-    }
-}
+struct Fwd5 {
+    double p[2], q[2];  // out = p x_s + q x_n, n the neighbour of the chirality's direction
+    int dir[2];
+    double mass, b;
+};
 
-template <typename R>
-__device__ void fwd_bidiag(cpx<R>* x, int Ls, R p, R q, int dir, R mass) {
-    if (dir == 0) {
-        cpx<R> last = x[Ls - 1];
-        for (int s = Ls - 1; s >= 1; s--) x[s] = p * x[s] + q * x[s - 1];
-        x[0] = p * x[0] - (q * mass) * last;
-    } else {
-        cpx<R> first = x[0];
-        for (int s = 0; s < Ls - 1; s++) x[s] = p * x[s] + q * x[s + 1];
-        x[Ls - 1] = p * x[Ls - 1] - (q * mass) * first;
-    }
-}
-
-template <int P>
-__global__ void op5_kernel(Geom g, Op5 op, int NS, const void* x, const void* y,
-                           void* out) {
-    typedef typename Field<P>::R R;
-    extern __shared__ __align__(128) unsigned char smraw[];
-    cpx<R>* sm = reinterpret_cast<cpx<R>*>(smraw);
-    const int Ls = g.Ls, LsP = g.Ls + 1;
-    long long n5 = (long long)g.Vh * Ls;
-    int j0 = blockIdx.x * NS;
-    int ns = min(NS, g.Vh - j0);
-    // stage: one thread per (site, s)
-    for (int idx = threadIdx.x; idx < ns * Ls; idx += blockDim.x) {
-        int lj = idx / Ls, s = idx - lj * Ls;
-        cpx<R> v[12];
-        Field<P>::load(x, j0 + lj, s, Ls, n5, v);
+__global__ void __launch_bounds__(256) fwd5_kernel(Geom g, Fwd5 o, const double2* __restrict__ x, const double2* y,
+                                                   double2* out) {
+    const long long n5 = (long long)g.Vh * g.Ls;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t >= n5) return;
+    const int Ls = g.Ls;
+    const long long j = t / Ls;
+    const int s = (int)(t - j * Ls);
+    const double2* xs = x + j * 12 * Ls;
+    double2* os = out + j * 12 * Ls;
 #pragma unroll
-        for (int c = 0; c < 12; c++) sm[(lj * 12 + c) * LsP + s] = v[c];
-    }
-    __syncthreads();
-    // columns: one thread per (site, component)
-    for (int idx = threadIdx.x; idx < ns * 12; idx += blockDim.x) {
-        int c = idx % 12;
-        int h = c < 6 ? 0 : 1;
-        cpx<R>* col = sm + idx * LsP;
-        if (op.inv[h]) inv_bidiag<R>(col, Ls, (R)op.p1[h], (R)op.q1[h], op.dir1[h], (R)op.mass);
-        cpx<R> d = mk(R(0), R(0));
-        bool r1 = op.sigma[h] != 0.0;
-        if (r1) {
-            const double* v = op.v[h];
-            for (int s = 0; s < Ls; s++) d = d + (R)__ldg(v + s) * col[s];
+    for (int h = 0; h < 2; h++) {
+        int n;
+        double q = o.q[h];
+        if (o.dir[h] == 0) {
+            n = s - 1;
+            if (n < 0) { n = Ls - 1; q *= -o.mass; }
+        } else {
+            n = s + 1;
+            if (n == Ls) { n = 0; q *= -o.mass; }
         }
-        if (op.fwd[h]) fwd_bidiag<R>(col, Ls, (R)op.p2[h], (R)op.q2[h], op.dir2[h], (R)op.mass);
-        if (r1) {
-            const double* w = op.w[h];
-            cpx<R> sd = (R)op.sigma[h] * d;
-            for (int s = 0; s < Ls; s++) col[s] = col[s] + (R)__ldg(w + s) * sd;
+        double2 a[6], b[6], c[6];
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            a[k] = __ldg(xs + (6 * h + k) * Ls + s);
+            b[k] = __ldg(xs + (6 * h + k) * Ls + n);
+            if (y) c[k] = __ldcs(y + (j * 12 + 6 * h + k) * Ls + s);
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            double re = fma(o.p[h], a[k].x, q * b[k].x), im = fma(o.p[h], a[k].y, q * b[k].y);
+            if (y) {
+                re = fma(o.b, c[k].x, re);
+                im = fma(o.b, c[k].y, im);
+            }
+            os[(6 * h + k) * Ls + s] = make_double2(re, im);
         }
     }
-    __syncthreads();
-    // write back: one thread per (site, s)
-    for (int idx = threadIdx.x; idx < ns * Ls; idx += blockDim.x) {
-        int lj = idx / Ls, s = idx - lj * Ls;
-        cpx<R> v[12];
-#pragma unroll
-        for (int c = 0; c < 12; c++) v[c] = (R)op.a_out * sm[(lj * 12 + c) * LsP + s];
-        if (y != nullptr && op.b_in != 0.0) {
-            cpx<R> yv[12];
-            Field<P>::load(y, j0 + lj, s, Ls, n5, yv);
-#pragma unroll
-            for (int c = 0; c < 12; c++) v[c] = v[c] + (R)op.b_in * yv[c];
-        }
-        Field<P>::store(out, j0 + lj, s, Ls, n5, v);
-    }
-}
-
-template <int P>
-void run_op5(const eofa_ctx* ctx, const Op5& op, const void* x, const void* y, void* out, cudaStream_t st) {
-    typedef typename Field<P>::R R;
-    Geom g = ctx_geom(ctx);
-    size_t per_site = (size_t)12 * (g.Ls + 1) * sizeof(cpx<R>);
-    int NS = (int)(24576 / per_site);
-    if (NS < 1) NS = 1;
-    if (NS > 32) NS = 32;
-    size_t smem = per_site * NS;
-    unsigned nb = (unsigned)((g.Vh + NS - 1) / NS);
-    if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(op5_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    prof_begin(ctx, 3 + P, st);
-    op5_kernel<P><<<nb, 128, smem, st>>>(g, op, NS, x, y, out);
-    EOFA_LAUNCHED();
-    prof_end(ctx, st);
 }
 
 }  // namespace
 
 void launch_op5(const eofa_ctx* ctx, int prec, const Op5& op, const void* x, const void* y, void* out,
                 cudaStream_t st) {
-    if (prec == P64) run_op5<P64>(ctx, op, x, y, out, st);
-    else if (prec == P32) run_op5<P32>(ctx, op, x, y, out, st);
-    else run_op5<P16>(ctx, op, x, y, out, st);
+    const void* yy = op.b_in != 0.0 ? y : nullptr;
+    const bool stencil = !op.inv[0] && !op.inv[1] && op.sigma[0] == 0.0 && op.sigma[1] == 0.0;
+    // (out = x in place goes through shared memory: the stencil's threads read each other's slices)
+    if (prec != P64 || !stencil || x == out) {
+        fused_local5(ctx, prec, op, x, nullptr, 0.0, nullptr, 0, 0, nullptr, out, op.a_out, nullptr, 0, st, yy, op.b_in);
+        return;
+    }
+    Fwd5 o;
+    for (int h = 0; h < 2; h++) {
+        o.p[h] = op.a_out * (op.fwd[h] ? op.p2[h] : 1.0);
+        o.q[h] = op.a_out * (op.fwd[h] ? op.q2[h] : 0.0);
+        o.dir[h] = op.dir2[h];
+    }
+    o.mass = op.mass;
+    o.b = op.b_in;
+    const Geom g = ctx_geom(ctx);
+    const long long n5 = (long long)g.Vh * g.Ls;
+    prof_begin(ctx, 3 + P64, st, (double)n5 * 192.0 * (yy ? 3.0 : 2.0));
+    fwd5_kernel<<<(unsigned)((n5 + 255) / 256), 256, 0, st>>>(g, o, (const double2*)x, (const double2*)yy, (double2*)out);
+    EOFA_LAUNCHED();
+    prof_end(ctx, st);
 }
