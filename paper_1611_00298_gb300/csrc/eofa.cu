@@ -18,6 +18,7 @@
 #include "api_util.h"
 
 #include <cmath>
+#include <cstdint>
 
 namespace {
 
@@ -43,6 +44,7 @@ __global__ void embed_kernel(long long V, int Ls, const double2* __restrict__ ph
 template <int MU>
 __device__ __forceinline__ void proj_A(const cpx<double>* v, int sg, cpx<double> out[6]) {
     // out = v_u + sg A_mu v_l (two spins x three colours)
+#pragma unroll
     for (int c = 0; c < 3; c++) {
         cpx<double> l0 = v[6 + c], l1 = v[9 + c], a0, a1;
         if (MU == 0) { a0 = mitimes(l1); a1 = mitimes(l0); }
@@ -54,94 +56,142 @@ __device__ __forceinline__ void proj_A(const cpx<double>* v, int sg, cpx<double>
     }
 }
 
-template <int MU>
-__device__ void accumulate_Y(const double2* chi, long long V, int Ls, long long i, long long ifw, double coef,
-                             cpx<double> Y[9]) {
-    for (int s = 0; s < Ls; s++) {
-        cpx<double> vf[12], vb[12], h[6], g[6];
-        const double2* pf = chi + ((long long)s * V + ifw) * 12;
-        const double2* pb = chi + ((long long)(Ls - 1 - s) * V + i) * 12;
-        for (int c = 0; c < 12; c++) {
-            vf[c] = mk(pf[c].x, pf[c].y);
-            vb[c] = mk(pb[c].x, pb[c].y);
+// the 12 components of one site and slice: 192 contiguous bytes, in 32-byte
+// loads (WIDE: whole sectors) or, for fields that start on a 16-byte boundary
+// only, in 16-byte ones
+template <bool WIDE>
+__device__ __forceinline__ void load_site(const double2* p, cpx<double> v[12]) {
+#pragma unroll
+    for (int c = 0; c < 12; c += 2) {
+        if (WIDE) {
+            asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                : "=d"(v[c].re), "=d"(v[c].im), "=d"(v[c + 1].re), "=d"(v[c + 1].im)
+                : "l"(p + c));
+        } else {
+            const double2 a = __ldg(p + c), b = __ldg(p + c + 1);
+            v[c] = mk(a.x, a.y);
+            v[c + 1] = mk(b.x, b.y);
         }
-        proj_A<MU>(vf, -1, h);
-        proj_A<MU>(vb, +1, g);
-        for (int b = 0; b < 3; b++)
-            for (int a = 0; a < 3; a++) {
-                cpx<double> acc = cjmul(g[a], h[b]);
-                acc = acc + cjmul(g[3 + a], h[3 + b]);
-                Y[3 * b + a] = Y[3 * b + a] + coef * acc;
-            }
     }
 }
 
+// Y += sum_s h(x + mu, s) g(x, Ls - 1 - s)^+ over the two half spins, as chains
+// of multiply-adds.  Four slices are summed before they are added to Y: 18
+// additions for 384 instructions, and a rounding error below that of adding
+// every product's sum to Y (one long chain had 1.5 times that).
+template <int MU, bool WIDE>
+__device__ __forceinline__ void accumulate_Y(const double2* chi, long long V, int Ls, long long i, long long ifw,
+                                             cpx<double> Y[9]) {
+    for (int s0 = 0; s0 < Ls; s0 += 4) {
+        cpx<double> T[9];
+#pragma unroll
+        for (int e = 0; e < 9; e++) T[e] = mk(0.0, 0.0);
+        const int n = min(4, Ls - s0);
+        for (int k = 0; k < n; k++) {
+            const int s = s0 + k;
+            cpx<double> v[12], h[6], g[6];
+            load_site<WIDE>(chi + ((long long)s * V + ifw) * 12, v);
+            proj_A<MU>(v, -1, h);
+            load_site<WIDE>(chi + ((long long)(Ls - 1 - s) * V + i) * 12, v);
+            proj_A<MU>(v, +1, g);
+#pragma unroll
+            for (int b = 0; b < 3; b++)
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    cpx<double> y = T[3 * b + a];
+#pragma unroll
+                    for (int q = 0; q < 2; q++) {  // conj(g) h
+                        const cpx<double> u = g[3 * q + a], w = h[3 * q + b];
+                        y.re = fma(u.re, w.re, y.re);
+                        y.im = fma(u.re, w.im, y.im);
+                        y.re = fma(u.im, w.im, y.re);
+                        y.im = fma(-u.im, w.re, y.im);
+                    }
+                    T[3 * b + a] = y;
+                }
+        }
+#pragma unroll
+        for (int e = 0; e < 9; e++) Y[e] = Y[e] + T[e];
+    }
+}
+
+template <int MU, bool WIDE>
+__device__ __forceinline__ void link_Y(const double2* chiL, const double2* chiR, long long V, int Ls, long long i,
+                                       long long ifw, double f, cpx<double> Y[9]) {
+    // Y_L - Y_R: a null chi drops its term (the force of S_L or S_R alone)
+    if (chiR) {
+        accumulate_Y<MU, WIDE>(chiR, V, Ls, i, ifw, Y);
+#pragma unroll
+        for (int e = 0; e < 9; e++) Y[e] = mk(-Y[e].re, -Y[e].im);
+    }
+    if (chiL) accumulate_Y<MU, WIDE>(chiL, V, Ls, i, ifw, Y);
+#pragma unroll
+    for (int e = 0; e < 9; e++) Y[e] = f * Y[e];
+}
+
 // mode 0: traceless Hermitian force F; mode 1: real-view gradient -Y^+
-__global__ void force_kernel(Coords d, int Ls, int bc_t, double k, const double2* __restrict__ U,
-                             const double2* __restrict__ chiL, const double2* __restrict__ chiR, double2* __restrict__ F,
-                             int mode) {
-    long long V = (long long)d.X * d.Y * d.Z * d.T;
-    long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= 4 * V) return;
-    long long i = t / 4;
-    int mu = (int)(t % 4);
-    int x = (int)(i % d.X), y = (int)((i / d.X) % d.Y), z = (int)((i / ((long long)d.X * d.Y)) % d.Z),
-        tt = (int)(i / ((long long)d.X * d.Y * d.Z));
-    int c[4] = {x, y, z, tt};
-    int n[4] = {d.X, d.Y, d.Z, d.T};
-    double phase = 1.0;
-    c[mu] += 1;
-    if (c[mu] == n[mu]) {
-        c[mu] = 0;
-        if (mu == 3) phase = (double)bc_t;
-    }
-    long long ifw = c[0] + (long long)d.X * (c[1] + (long long)d.Y * (c[2] + (long long)d.Z * c[3]));
+//
+// Bound by the FP64 pipe: 24 additions for the half spinors, 72 multiply-adds
+// for the outer product and 4.5 additions of partial sums per link, slice and
+// chi (24^3 x 32 x 24: 8.5e9 of them, 16 ms at the measured 1.057 TFLOP/s).  A block works on one
+// direction (the four blocks of a run of sites are neighbours in the grid and
+// share their spinors in L2): with the four directions in the lanes of a warp,
+// as before, every warp ran all four one after another, and with products
+// added and scaled one by one 150 instructions a term, it took 82.1 ms there;
+// this form 15.2 ms.
+template <int NT, bool WIDE>
+__global__ void __launch_bounds__(NT) force_kernel(Coords d, int Ls, int bc_t, double k, const double2* __restrict__ U,
+                                                   const double2* __restrict__ chiL, const double2* __restrict__ chiR,
+                                                   double2* __restrict__ F, int mode) {
+    const long long V = (long long)d.X * d.Y * d.Z * d.T;
+    const int mu = blockIdx.x & 3;
+    const long long i = (blockIdx.x >> 2) * (long long)NT + threadIdx.x;
+    if (i >= V) return;
+    const int x = (int)(i % d.X), y = (int)((i / d.X) % d.Y), z = (int)((i / ((long long)d.X * d.Y)) % d.Z),
+              tt = (int)(i / ((long long)d.X * d.Y * d.Z));
+    const int fx = mu == 0 ? (x + 1 == d.X ? 0 : x + 1) : x, fy = mu == 1 ? (y + 1 == d.Y ? 0 : y + 1) : y;
+    const int fz = mu == 2 ? (z + 1 == d.Z ? 0 : z + 1) : z, ft = mu == 3 ? (tt + 1 == d.T ? 0 : tt + 1) : tt;
+    const double phase = mu == 3 && tt + 1 == d.T ? (double)bc_t : 1.0;
+    const long long ifw = fx + (long long)d.X * (fy + (long long)d.Y * (fz + (long long)d.Z * ft));
     cpx<double> Y[9];
+#pragma unroll
     for (int e = 0; e < 9; e++) Y[e] = mk(0.0, 0.0);
-    switch (mu) {
-        // a null chi drops its term (the force of S_L or S_R alone)
-        case 0:
-            if (chiL) accumulate_Y<0>(chiL, V, Ls, i, ifw, k, Y);
-            if (chiR) accumulate_Y<0>(chiR, V, Ls, i, ifw, -k, Y);
-            break;
-        case 1:
-            if (chiL) accumulate_Y<1>(chiL, V, Ls, i, ifw, k, Y);
-            if (chiR) accumulate_Y<1>(chiR, V, Ls, i, ifw, -k, Y);
-            break;
-        case 2:
-            if (chiL) accumulate_Y<2>(chiL, V, Ls, i, ifw, k, Y);
-            if (chiR) accumulate_Y<2>(chiR, V, Ls, i, ifw, -k, Y);
-            break;
-        default:
-            if (chiL) accumulate_Y<3>(chiL, V, Ls, i, ifw, k, Y);
-            if (chiR) accumulate_Y<3>(chiR, V, Ls, i, ifw, -k, Y);
-            break;
-    }
-    for (int e = 0; e < 9; e++) Y[e] = phase * Y[e];
-    double2* out = F + t * 9;
+    const double f = phase * k;
+    if (mu == 0) link_Y<0, WIDE>(chiL, chiR, V, Ls, i, ifw, f, Y);
+    else if (mu == 1) link_Y<1, WIDE>(chiL, chiR, V, Ls, i, ifw, f, Y);
+    else if (mu == 2) link_Y<2, WIDE>(chiL, chiR, V, Ls, i, ifw, f, Y);
+    else link_Y<3, WIDE>(chiL, chiR, V, Ls, i, ifw, f, Y);
+    const long long l = i * 4 + mu;
+    double2* out = F + l * 9;
     if (mode == 1) {
+#pragma unroll
         for (int a = 0; a < 3; a++)
+#pragma unroll
             for (int b = 0; b < 3; b++) out[3 * a + b] = make_double2(-Y[3 * b + a].re, Y[3 * b + a].im);
         return;
     }
-    const double2* u = U + t * 9;
+    const double2* u = U + l * 9;
     cpx<double> X[9];
+#pragma unroll
     for (int a = 0; a < 3; a++)
+#pragma unroll
         for (int b = 0; b < 3; b++) {
             cpx<double> acc = mk(0.0, 0.0);
+#pragma unroll
             for (int e = 0; e < 3; e++) acc = acc + cmul(mk(u[3 * a + e].x, u[3 * a + e].y), Y[3 * e + b]);
             X[3 * a + b] = acc;
         }
     // A = X - X^+ (anti-Hermitian), F = -(i/4)(A - tr(A)/3)
     cpx<double> A[9];
+#pragma unroll
     for (int a = 0; a < 3; a++)
+#pragma unroll
         for (int b = 0; b < 3; b++) A[3 * a + b] = X[3 * a + b] - mk(X[3 * b + a].re, -X[3 * b + a].im);
-    cpx<double> tr3 = (1.0 / 3.0) * (A[0] + A[4] + A[8]);
+    const cpx<double> tr3 = (1.0 / 3.0) * (A[0] + A[4] + A[8]);
+#pragma unroll
     for (int a = 0; a < 3; a++) A[4 * a] = A[4 * a] - tr3;
-    for (int e = 0; e < 9; e++) {
-        cpx<double> f = mk(0.25 * A[e].im, -0.25 * A[e].re);  // -(i/4) A
-        out[e] = make_double2(f.re, f.im);
-    }
+#pragma unroll
+    for (int e = 0; e < 9; e++) out[e] = make_double2(0.25 * A[e].im, -0.25 * A[e].re);  // -(i/4) A
 }
 
 // U <- exp(i eps P) U, exp by Taylor series with scaling and squaring
@@ -305,9 +355,11 @@ static void launch_force(eofa_ctx* ctx, double k, const double* chiL, const doub
     require_gauge(ctx);
     Coords d = {ctx->dims[0], ctx->dims[1], ctx->dims[2], ctx->dims[3]};
     const double* U = (const double*)ctx_buffer(ctx, "U", 0);
-    long long nl = 4LL * ctx->V;
-    force_kernel<<<nblk(nl, 128), 128, 0, st>>>(d, ctx->Ls, ctx->bc_t, k, (const double2*)U, (const double2*)chiL,
-                                                (const double2*)chiR, (double2*)F, mode);
+    constexpr int NT = 64;
+    const bool wide = !(((uintptr_t)chiL | (uintptr_t)chiR) & 31);
+    auto kern = wide ? force_kernel<NT, true> : force_kernel<NT, false>;
+    kern<<<4 * nblk(ctx->V, NT), NT, 0, st>>>(d, ctx->Ls, ctx->bc_t, k, (const double2*)U, (const double2*)chiL,
+                                             (const double2*)chiR, (double2*)F, mode);
     EOFA_LAUNCHED();
 }
 
