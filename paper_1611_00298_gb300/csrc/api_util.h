@@ -25,3 +25,7 @@ void gauge_force_launch(eofa_ctx* ctx, const double* U, double beta, int accumul
 extern "C" int eofa_force_parts_dev(eofa_ctx* ctx, int Ls, double alpha, double M5, double m1, double m2,
                                     int precision, double tol, const double* phi_dev, double* FL_dev, double* FR_dev,
                                     eofa_solve_info info[2], void* stream);
+// Uout <- exp(i eps P) Uin on canonical links (eofa.cu; Uout may be Uin), and to Ux if not null; the
+// packed links of the context are left as they are
+void link_update_launch(eofa_ctx* ctx, double eps, const double* P, const double* Uin, double* Uout, double* Ux,
+                        cudaStream_t st);

@@ -222,8 +222,9 @@ __constant__ double inv_factorial[19] = {
     1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
     1.0 / 20922789888000.0, 1.0 / 355687428096000.0, 1.0 / 6402373705728000.0};
 
+// Uout <- exp(i eps P) Uin (Uout may be Uin), and to Ux as well if given
 __global__ void __launch_bounds__(128) link_update_kernel(long long nlinks, double eps, const double2* __restrict__ P,
-                                                          double2* Uc, double2* Ux) {
+                                                          const double2* Uin, double2* Uout, double2* Ux) {
     const long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (l >= nlinks) return;
     cpx<double> A[9], A2[9], E[9];
@@ -269,11 +270,11 @@ __global__ void __launch_bounds__(128) link_update_kernel(long long nlinks, doub
         for (int e = 0; e < 9; e++) E[e] = A2[e];
     }
 #pragma unroll
-    for (int e = 0; e < 9; e++) A[e] = mk(Uc[l * 9 + e].x, Uc[l * 9 + e].y);
+    for (int e = 0; e < 9; e++) A[e] = mk(Uin[l * 9 + e].x, Uin[l * 9 + e].y);
     mat3_mul(E, A, A2);
 #pragma unroll
     for (int e = 0; e < 9; e++) {
-        Uc[l * 9 + e] = make_double2(A2[e].re, A2[e].im);
+        Uout[l * 9 + e] = make_double2(A2[e].re, A2[e].im);
         if (Ux) Ux[l * 9 + e] = make_double2(A2[e].re, A2[e].im);
     }
 }
@@ -343,6 +344,14 @@ ChiBufs eofa_chis(eofa_ctx* ctx, int Ls, double alpha, double M5, double m1, dou
 }
 
 }  // namespace
+
+void link_update_launch(eofa_ctx* ctx, double eps, const double* P, const double* Uin, double* Uout, double* Ux,
+                        cudaStream_t st) {
+    const long long nl = 4LL * ctx->V;
+    link_update_kernel<<<nblk(nl, 128), 128, 0, st>>>(nl, eps, (const double2*)P, (const double2*)Uin, (double2*)Uout,
+                                                      (double2*)Ux);
+    EOFA_LAUNCHED();
+}
 
 void eofa_embed(eofa_ctx* ctx, const double* phi, const double* Om_dev, int chi, double* out, cudaStream_t st) {
     long long V = ctx->V, n = V * 12 * ctx->Ls;
@@ -487,9 +496,7 @@ int eofa_link_update_dev(eofa_ctx* ctx, double eps, const double* P_dev, double*
     try {
         require_gauge(ctx);
         double* Uc = (double*)ctx_buffer(ctx, "U", 0);
-        long long nl = 4LL * ctx->V;
-        link_update_kernel<<<nblk(nl, 128), 128, 0, st>>>(nl, eps, (const double2*)P_dev, (double2*)Uc, (double2*)U_dev);
-        EOFA_LAUNCHED();
+        link_update_launch(ctx, eps, P_dev, Uc, Uc, U_dev, st);
         launch_gauge_pack(ctx, Uc, st);
     } catch (const eofa_error& e) {
         return fail(ctx, e.code, e.msg);
