@@ -7,8 +7,9 @@
 // form a group (at most MR_MAX systems); a system on a large lattice is a
 // group of its own (MR_SINGLE_SITES).  A group iterates its systems in lock
 // step with the multi-system kernels of mrhs.cuh: the five-launch form of
-// the CG iteration of solver.cu, each launch for all of them, each link row
-// and neighbour index fetched once for the whole group.  The CG loop of a group runs on the device: a CUDA graph
+// the CG iteration of solver.cu, each launch for all of them (FP32 and FP16
+// storage, even Ls: one grid row a system, the rows sharing links through the
+// caches; else one block for several systems).  The CG loop of a group runs on the device: a CUDA graph
 // holds one WHILE conditional node whose body is K CG iterations of every
 // active system followed by a one-block decision kernel; the kernel reads
 // each system's |r|^2 and keeps the loop going until some system has
@@ -76,10 +77,12 @@ __global__ void mr_decide_kernel(MRPtrs a, int nr, double* ctl, cudaGraphConditi
     if (threadIdx.x == 0) cudaGraphSetConditional(h, stop ? 0u : 1u);
 }
 
-void mr_dslash(const eofa_ctx* ctx, int prec, int par, int dag, int mode, const MRPtrs& a, const Op5* ops,
-               const Op5* ops2, int nr, bool hasop, double a_out, double b_in, int slot, int it, int slot2,
-               cudaStream_t st) {
-    if (prec == P64) mr_dslash_p64(ctx, par, dag, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st);
+void mr_dslash(const eofa_ctx* ctx, int prec, int par, int dag, int mode, const MRPtrs& a, const void* pops,
+               const Op5* ops, const Op5* ops2, int nr, bool hasop, double a_out, double b_in, int slot, int it,
+               int slot2, cudaStream_t st) {
+    if (pops && prec == P32) mr_pair_p32(ctx, par, dag, mode, a, pops, ops, ops2, nr, a_out, b_in, slot, it, slot2, st);
+    else if (pops) mr_pair_p16(ctx, par, dag, mode, a, pops, ops, ops2, nr, a_out, b_in, slot, it, slot2, st);
+    else if (prec == P64) mr_dslash_p64(ctx, par, dag, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st);
     else if (prec == P32) mr_dslash_p32(ctx, par, dag, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st);
     else mr_dslash_p16(ctx, par, dag, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st);
 }
@@ -99,6 +102,8 @@ struct Group {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t done = nullptr;
+    void* pops = nullptr;        // device: the blocks as the two-slice kernels take them
+    bool pairs = false;          // the captured set runs on those kernels
     Op5* ops = nullptr;          // device: [Gi x MR_MAX][GiT x MR_MAX] of the captured set
     double* ctl = nullptr;       // device control block
     double* ctl_host = nullptr;  // pinned mirror
@@ -128,13 +133,14 @@ void enqueue_group_iteration(Group& g, std::vector<Solve>& sv, int it, cudaStrea
     }
     const Op5* Gi = g.ops;
     const Op5* GiT = g.ops + MR_MAX;
+    const void* po = g.pairs ? g.pops : nullptr;
     // q = A p: te = G'^-1 D_eo p; q = p - G'^-1 D_oe te, |q|^2 -> delta, to = G'^-T q
-    mr_dslash(g.ctx, g.prec, 0, 0, 0, k1, Gi, GiT, n, true, 1.0, 0.0, -1, it, -1, st);
-    mr_dslash(g.ctx, g.prec, 1, 0, 1, k2, Gi, GiT, n, true, -1.0, 1.0, SC_DELTA, it, -1, st);
+    mr_dslash(g.ctx, g.prec, 0, 0, 0, k1, po, Gi, GiT, n, true, 1.0, 0.0, -1, it, -1, st);
+    mr_dslash(g.ctx, g.prec, 1, 0, 1, k2, po, Gi, GiT, n, true, -1.0, 1.0, SC_DELTA, it, -1, st);
     // s -= alpha A^+ q: te = G'^-T D^+_eo to; s -= alpha (q - D^+_oe te), |s|^2 -> gamma (next
     // parity); r -= alpha q, |r|^2 -> ring
-    mr_dslash(g.ctx, g.prec, 0, 1, 0, k4, GiT, GiT, n, true, 1.0, 0.0, -1, it, -1, st);
-    mr_dslash(g.ctx, g.prec, 1, 1, 2, k5, GiT, GiT, n, false, -1.0, 1.0, SC_GAMMA + ((it + 1) & 1), it,
+    mr_dslash(g.ctx, g.prec, 0, 1, 0, k4, po, GiT, GiT, n, true, 1.0, 0.0, -1, it, -1, st);
+    mr_dslash(g.ctx, g.prec, 1, 1, 2, k5, po, GiT, GiT, n, false, -1.0, 1.0, SC_GAMMA + ((it + 1) & 1), it,
               SC_RRH + (it % MR_BODY), st);
     // x += alpha p; p = s + beta p
     mr_xp(g.ctx, g.prec, k6, n, it, st);
@@ -162,6 +168,9 @@ void build_graph(Group& g, std::vector<Solve>& sv, const std::vector<int>& activ
         h[MR_MAX + a] = op_finalize(sv[active[a]].GiT, g.ctx->Ls);
     }
     EOFA_CUDA(cudaMemcpyAsync(g.ops, h.data(), h.size() * sizeof(Op5), cudaMemcpyHostToDevice, g.st));
+    std::vector<char> hp(mr_pair_ops_bytes());
+    g.pairs = g.prec != P64 && !g.single && mr_pair_ops_fill(h.data(), h.data() + MR_MAX, n, g.ctx->Ls, hp.data());
+    if (g.pairs) EOFA_CUDA(cudaMemcpyAsync(g.pops, hp.data(), hp.size(), cudaMemcpyHostToDevice, g.st));
     EOFA_CUDA(cudaStreamSynchronize(g.st));
     EOFA_CUDA(cudaGraphCreate(&g.graph, 0));
     cudaGraphConditionalHandle handle;
@@ -315,6 +324,7 @@ extern "C" int eofa_solve_batched(eofa_ctx* const* ctxs, int n, const eofa_solve
                 EOFA_CUDA(cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming));
                 const std::string gt = "_g" + std::to_string(groups.size() - 1);
                 g->ops = (Op5*)ctx_buffer(g->ctx, "bt_ops" + gt, 2 * MR_MAX * sizeof(Op5));
+                g->pops = ctx_buffer(g->ctx, "bt_pops" + gt, mr_pair_ops_bytes());
                 g->ctl = (double*)ctx_buffer(g->ctx, "bt_ctl" + gt, CTL_DOUBLES * sizeof(double));
                 EOFA_CUDA(cudaMallocHost((void**)&g->ctl_host, CTL_DOUBLES * sizeof(double)));
                 open[key] = g;

@@ -38,7 +38,10 @@
 // tiles dealt so that each half of the SMs sweeps its own half of t 0.68.
 #pragma once
 #include "dslash_impl.cuh"
+#include "mrhs.h"
 
+#include <algorithm>
+#include <climits>
 #include <cmath>
 
 #define PAIR_THREADS 96
@@ -428,8 +431,8 @@ __device__ __forceinline__ void pair_op(const PairOp& o, int NS, int nsites, int
         pair_ends<!UP, 1>(o, pl, Ls, ls, sp, sm, wv, v);
     }
     __syncthreads();
-    // half of the threads (48: one and a half warps) take the columns of each chirality
-    const int half = PAIR_THREADS / 2, hh = threadIdx.x >= half;
+    // half of the threads take the columns of each chirality
+    const int half = blockDim.x / 2, hh = threadIdx.x >= half;
     for (int idx = threadIdx.x - hh * half; idx < nsites * 6; idx += half) {
         const int site = idx / 6, c = idx - site * 6;
         cpx<float>* e = sm + pl.carry + (site * 12 + 6 * hh + c) * pl.lhp;
@@ -447,10 +450,9 @@ __device__ __forceinline__ void pair_op(const PairOp& o, int NS, int nsites, int
 
 // ---------------------------------------------------------------- kernel
 
+// the outputs beside the first, as in Epi
 struct EpiPair {
-    PairOp op2;
-    Op5 r2;            // MODE 1: op2's rank-one vectors
-    void* out2;        // as in Epi
+    void* out2;
     const void* aux;
     void* out3;
     const void* aux2;
@@ -463,17 +465,19 @@ struct ZBlocks {
     int n, tiles;
 };
 
+// One launch of one system.  r1, r2: the blocks whose rank-one vectors go with op, op2.
 template <int P, int DAG, int LS, bool HASOP, int MODE>
-__global__ void __launch_bounds__(PAIR_THREADS, 4)
-    dslash_pair_kernel(Geom g, int par, const void* __restrict__ in, void* out, const void* __restrict__ gauge, PairOp op,
-                       Op5 r1, const void* y, float a_out, float b_in, double* red, int slot, int NS, ZBlocks zb, EpiPair ep) {
+__device__ __forceinline__ void pair_body(const Geom& g, int par, const void* __restrict__ in, void* out,
+                                          const void* __restrict__ gauge, const PairOp& op, const Op5& r1,
+                                          const PairOp& op2, const Op5& r2, const void* y, float a_out, float b_in,
+                                          double* red, int slot, int NS, const ZBlocks& zb, const EpiPair& ep) {
     extern __shared__ __align__(128) unsigned char smraw[];
     constexpr int LH = LS / 2;
     const int Ls = LS > 0 ? LS : g.Ls, lh = Ls / 2;
     __shared__ float wv_s[HASOP ? 4 * EOFA_MAX_LS : 1];
     __shared__ float wv2_s[MODE == 1 ? 4 * EOFA_MAX_LS : 1];
     if (HASOP) stage_wv<float>(r1, Ls, wv_s);
-    if (MODE == 1) stage_wv<float>(ep.r2, Ls, wv2_s);
+    if (MODE == 1) stage_wv<float>(r2, Ls, wv2_s);
     if (HASOP || MODE == 1) __syncthreads();
     const float cz = MODE == 2 ? (float)(-cg_alpha(red, ep.it)) : 0.f;
     const float ax = MODE == 3 ? (float)cg_alpha(red, ep.it) : 0.f;
@@ -579,7 +583,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 4)
         }
         if (MODE == 1) {
             __syncthreads();  // the first block's carries are still being read
-            pair_op<LH, DAG != 0>(ep.op2, NS, nsites, ls, sp, lh, ok, smraw, wv2_s, v);
+            pair_op<LH, DAG != 0>(op2, NS, nsites, ls, sp, lh, ok, smraw, wv2_s, v);
             if (ok) Pair<P>::store(ep.out2, j, sp, Ls, n5, v);
         }
         if (HASOP) __syncthreads();
@@ -590,6 +594,36 @@ __global__ void __launch_bounds__(PAIR_THREADS, 4)
         if (MODE == 2 && ep.out2 != nullptr) grid_sum2(nacc, nacc2, red, slot, ep.slot2);
         else grid_sum(nacc, red, slot);
     }
+}
+
+template <int P, int DAG, int LS, bool HASOP, int MODE>
+__global__ void __launch_bounds__(PAIR_THREADS, 4)
+    dslash_pair_kernel(Geom g, int par, const void* __restrict__ in, void* out, const void* __restrict__ gauge, PairOp op,
+                       Op5 r1, PairOp op2, Op5 r2, const void* y, float a_out, float b_in, double* red, int slot, int NS,
+                       ZBlocks zb, EpiPair ep) {
+    pair_body<P, DAG, LS, HASOP, MODE>(g, par, in, out, gauge, op, r1, op2, r2, y, a_out, b_in, red, slot, NS, zb,
+                                              ep);
+}
+
+// The same launch for several systems on one lattice: system blockIdx.y, its
+// fields and scratch in a, its blocks in ops, ops2 (and r1, r2).
+template <int P, int DAG, int LS, bool HASOP, int MODE>
+__global__ void __launch_bounds__(PAIR_THREADS, 4)
+    mr_pair_kernel(Geom g, int par, MRPtrs a, const void* __restrict__ gauge, const PairOp* __restrict__ ops,
+                   const Op5* __restrict__ r1, const PairOp* __restrict__ ops2, const Op5* __restrict__ r2, float a_out,
+                   float b_in, int slot, int NS, ZBlocks zb, int it, int slot2) {
+    const int r = blockIdx.y;
+    __shared__ PairOp op_s, op2_s;
+    if (HASOP) {
+        for (int i = threadIdx.x; i < (int)(sizeof(PairOp) / 4); i += blockDim.x) {
+            reinterpret_cast<unsigned*>(&op_s)[i] = reinterpret_cast<const unsigned*>(ops + r)[i];
+            if (MODE == 1) reinterpret_cast<unsigned*>(&op2_s)[i] = reinterpret_cast<const unsigned*>(ops2 + r)[i];
+        }
+        __syncthreads();
+    }
+    EpiPair ep = {a.out2[r], nullptr, nullptr, nullptr, it, slot2};
+    pair_body<P, DAG, LS, HASOP, MODE>(g, par, a.in[r], a.out[r], gauge, op_s, r1[r], op2_s, r2[r], a.y[r], a_out, b_in,
+                                       a.red[r], slot, NS, zb, ep);
 }
 
 // ---------------------------------------------------------------- launch
@@ -631,29 +665,42 @@ inline ZBlocks z_blocks(const Geom& g, int NS, int spinor) {
     return ZBlocks{1, 0};
 }
 
+// block shape of a launch: sites, threads, dynamic shared memory
+struct PairShape {
+    int NS, threads;
+    size_t smem;
+};
+inline PairShape pair_shape(int Ls, bool hasop) {
+    PairShape p;
+    p.threads = PAIR_THREADS;
+    p.NS = PAIR_THREADS / (Ls / 2);
+    p.smem = hasop ? column_plan(p.NS, Ls).bytes : 0;
+    return p;
+}
+
 template <int P, int DAG, int LS, bool HASOP, int MODE>
-void launch_pair(const eofa_ctx* ctx, int par, const PairArgs& a, const PairOp& o, const EpiPair& e, cudaStream_t st) {
+void launch_pair(const eofa_ctx* ctx, int par, const PairArgs& a, const PairOp& o, const PairOp& o2, const EpiPair& e,
+                 cudaStream_t st) {
     Geom g = ctx_geom(ctx);
-    const int NS = PAIR_THREADS / (g.Ls / 2);
-    const size_t smem = HASOP ? column_plan(NS, g.Ls).bytes : 0;
+    const PairShape s = pair_shape(g.Ls, HASOP);
     auto k = dslash_pair_kernel<P, DAG, LS, HASOP, MODE>;
-    const unsigned grid = grid_size(k, PAIR_THREADS, smem, (g.Vh + NS - 1) / NS, ctx->sms);
-    k<<<grid, PAIR_THREADS, smem, st>>>(g, par, a.in, a.out, ctx->gauge[P32], o, a.op ? *a.op : Op5(), a.y, (float)a.a_out,
-                                        (float)a.b_in, a.red, a.slot, NS,
-                                        z_blocks(g, NS, P == P16 ? 52 : 96), e);
+    const unsigned grid = grid_size(k, s.threads, s.smem, (g.Vh + s.NS - 1) / s.NS, ctx->sms);
+    k<<<grid, s.threads, s.smem, st>>>(g, par, a.in, a.out, ctx->gauge[P32], o, a.op ? *a.op : Op5(), o2,
+                                       a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
+                                       z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
     EOFA_LAUNCHED();
 }
 
 template <int P, int LS>
-void launch_pair_ls(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, const PairOp& o, const EpiPair& e,
-                    cudaStream_t st) {
-    if (a.mode == 1) launch_pair<P, 0, LS, true, 1>(ctx, par, a, o, e, st);
-    else if (a.mode == 2) launch_pair<P, 1, LS, false, 2>(ctx, par, a, o, e, st);
-    else if (a.mode == 3) launch_pair<P, 1, LS, true, 3>(ctx, par, a, o, e, st);
-    else if (a.op && dag) launch_pair<P, 1, LS, true, 0>(ctx, par, a, o, e, st);
-    else if (a.op) launch_pair<P, 0, LS, true, 0>(ctx, par, a, o, e, st);
-    else if (dag) launch_pair<P, 1, LS, false, 0>(ctx, par, a, o, e, st);
-    else launch_pair<P, 0, LS, false, 0>(ctx, par, a, o, e, st);
+void launch_pair_ls(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, const PairOp& o, const PairOp& o2,
+                    const EpiPair& e, cudaStream_t st) {
+    if (a.mode == 1) launch_pair<P, 0, LS, true, 1>(ctx, par, a, o, o2, e, st);
+    else if (a.mode == 2) launch_pair<P, 1, LS, false, 2>(ctx, par, a, o, o2, e, st);
+    else if (a.mode == 3) launch_pair<P, 1, LS, true, 3>(ctx, par, a, o, o2, e, st);
+    else if (a.op && dag) launch_pair<P, 1, LS, true, 0>(ctx, par, a, o, o2, e, st);
+    else if (a.op) launch_pair<P, 0, LS, true, 0>(ctx, par, a, o, o2, e, st);
+    else if (dag) launch_pair<P, 1, LS, false, 0>(ctx, par, a, o, o2, e, st);
+    else launch_pair<P, 0, LS, false, 0>(ctx, par, a, o, o2, e, st);
 }
 
 template <int P>
@@ -664,27 +711,62 @@ bool pair_dslash(const eofa_ctx* ctx, int par, int dag, const PairArgs& a, cudaS
     if ((a.mode == 1 && dag) || (a.mode >= 2 && !dag)) return false;
     for (const void* q : {a.in, (const void*)a.out, a.y, (const void*)a.out2, a.aux, (const void*)a.out3, a.aux2})
         if ((uintptr_t)q & 31) return false;
-    PairOp o = {};
-    EpiPair e = {};
+    PairOp o = {}, o2 = {};
     if (a.op && !pair_op_of(*a.op, Ls, dag == 0, -0.5 * a.a_out, o)) return false;
-    if (a.op2) {
-        if (!pair_op_of(*a.op2, Ls, dag != 0, 1.0, e.op2)) return false;
-        e.r2 = *a.op2;
-    }
-    e.out2 = a.out2;
-    e.aux = a.aux;
-    e.out3 = a.out3;
-    e.aux2 = a.aux2;
-    e.it = a.it;
-    e.slot2 = a.slot2;
+    if (a.op2 && !pair_op_of(*a.op2, Ls, dag != 0, 1.0, o2)) return false;
+    const EpiPair e = {a.out2, a.aux, a.out3, a.aux2, a.it, a.slot2};
     switch (Ls) {
-        case 8: launch_pair_ls<P, 8>(ctx, par, dag, a, o, e, st); break;
-        case 12: launch_pair_ls<P, 12>(ctx, par, dag, a, o, e, st); break;
-        case 16: launch_pair_ls<P, 16>(ctx, par, dag, a, o, e, st); break;
-        case 24: launch_pair_ls<P, 24>(ctx, par, dag, a, o, e, st); break;
-        default: launch_pair_ls<P, 0>(ctx, par, dag, a, o, e, st); break;
+        case 8: launch_pair_ls<P, 8>(ctx, par, dag, a, o, o2, e, st); break;
+        case 12: launch_pair_ls<P, 12>(ctx, par, dag, a, o, o2, e, st); break;
+        case 16: launch_pair_ls<P, 16>(ctx, par, dag, a, o, o2, e, st); break;
+        case 24: launch_pair_ls<P, 24>(ctx, par, dag, a, o, o2, e, st); break;
+        default: launch_pair_ls<P, 0>(ctx, par, dag, a, o, o2, e, st); break;
     }
     return true;
+}
+
+// ---------------------------------------------------------------- several systems
+
+template <int P, int DAG, int LS, bool HASOP, int MODE>
+void launch_mr_pair(const eofa_ctx* ctx, int par, const MRPtrs& a, const PairOp* ops, const Op5* r1, const PairOp* ops2,
+                    const Op5* r2, int nr, double a_out, double b_in, int slot, int it, int slot2, cudaStream_t st) {
+    Geom g = ctx_geom(ctx);
+    const PairShape s = pair_shape(g.Ls, HASOP);
+    const int ntiles = (g.Vh + s.NS - 1) / s.NS;
+    auto k = mr_pair_kernel<P, DAG, LS, HASOP, MODE>;
+    const int all = (int)grid_size(k, s.threads, s.smem, INT_MAX, ctx->sms);  // resident blocks, over the systems
+    const int gx = std::max(1, std::min(ntiles, (all + nr - 1) / nr));
+    k<<<dim3(gx, nr), s.threads, s.smem, st>>>(g, par, a, ctx->gauge[P32], ops, r1, ops2, r2, (float)a_out, (float)b_in, slot,
+                                              s.NS, z_blocks(g, s.NS, P == P16 ? 52 : 96), it, slot2);
+    EOFA_LAUNCHED();
+}
+
+// The launches of the lock-step iteration (batch.cu): blocks by kind, MR_MAX systems each
+// (0: G'^-1 of te = G'^-1 D p, 1: of q = p - G'^-1 D te, 2: G'^-T of te = G'^-T D^+ to, 3: of to = G'^-T q).
+template <int P, int LS>
+void mr_pair_ls(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a, const PairOp* po, const Op5* ops,
+                const Op5* ops2, int nr, double a_out, double b_in, int slot, int it, int slot2, cudaStream_t st) {
+    if (mode == 1)
+        launch_mr_pair<P, 0, LS, true, 1>(ctx, par, a, po + MR_MAX, ops, po + 3 * MR_MAX, ops2, nr, a_out, b_in, slot, it,
+                                          slot2, st);
+    else if (mode == 2)
+        launch_mr_pair<P, 1, LS, false, 2>(ctx, par, a, po, ops, po, ops2, nr, a_out, b_in, slot, it, slot2, st);
+    else if (dag)
+        launch_mr_pair<P, 1, LS, true, 0>(ctx, par, a, po + 2 * MR_MAX, ops, po, ops2, nr, a_out, b_in, slot, it, slot2, st);
+    else
+        launch_mr_pair<P, 0, LS, true, 0>(ctx, par, a, po, ops, po, ops2, nr, a_out, b_in, slot, it, slot2, st);
+}
+
+template <int P>
+void mr_pair(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a, const void* pops, const Op5* ops,
+             const Op5* ops2, int nr, double a_out, double b_in, int slot, int it, int slot2, cudaStream_t st) {
+    const PairOp* po = (const PairOp*)pops;
+    switch (ctx->Ls) {
+        case 8: mr_pair_ls<P, 8>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
+        case 12: mr_pair_ls<P, 12>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
+        case 16: mr_pair_ls<P, 16>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
+        default: mr_pair_ls<P, 0>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
+    }
 }
 
 }  // namespace

@@ -45,3 +45,15 @@ __host__ __device__ inline size_t mr_head_bytes(int RB, int Ls) {
 MR_DECLARE(p64)
 MR_DECLARE(p32)
 MR_DECLARE(p16)
+
+// The lock-step launches on the two-slices-per-thread kernels (dslash_pair.cuh; FP32 and FP16 storage, even Ls):
+// the same modes and arguments, and pops, a device array of mr_pair_ops_bytes() that mr_pair_ops_fill has
+// prepared from n finalised blocks (false: a block is not of the form they take).
+size_t mr_pair_ops_bytes();
+bool mr_pair_ops_fill(const Op5* Gi, const Op5* GiT, int n, int Ls, void* host);
+#define MR_PAIR_DECLARE(NAME)                                                                                  \
+    void mr_pair_##NAME(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a, const void* pops,   \
+                        const Op5* ops, const Op5* ops2, int nr, double a_out, double b_in, int slot, int it, \
+                        int slot2, cudaStream_t st);
+MR_PAIR_DECLARE(p32)
+MR_PAIR_DECLARE(p16)
