@@ -23,6 +23,9 @@
 
 #include <cstdio>
 #include <cstdlib>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include <type_traits>
 
 // minimum resident blocks of 256 threads per SM requested from the register
@@ -693,6 +696,7 @@ template <int P, int DAG, int LS, bool HASOP, int SPT, int MODE = 0>
 __global__ void __launch_bounds__(256, SPT == 2 ? 2 : (MODE == 1 ? EOFA_MODE1_MINB : (HASOP ? EOFA_DSLASH_MINB : EOFA_HOP_MINB))) dslash_kernel(
     Geom g, int par, const void* __restrict__ in, void* out, const void* __restrict__ gauge, Op5 op, const void* y,
     double a_out, double b_in, double* red, int slot, int NS, Epi ep) {
+    chain_wait();
     typedef typename Field<P>::R R;
     extern __shared__ __align__(128) unsigned char smraw[];
     cpx<R>* sm = reinterpret_cast<cpx<R>*>(smraw);
@@ -863,6 +867,7 @@ __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, O
                                                      const double* sc, int it, int use_alpha, void* xw, void* out,
                                                      double a_out, const void* y, double b_in, double* red, int slot,
                                                      int NS) {
+    chain_wait();
     typedef typename Field<P>::R R;
     extern __shared__ __align__(128) unsigned char smraw[];
     cpx<R>* sm = reinterpret_cast<cpx<R>*>(smraw);
@@ -941,6 +946,7 @@ __global__ void __launch_bounds__(256, EOFA_LOCAL5_MINB) local5_kernel(Geom g, O
 template <int P, int PX>
 __global__ void __launch_bounds__(256) xp_update_kernel(Geom g, const double* sc, int it, void* x, void* p,
                                                         const void* s) {
+    chain_wait();
     typedef typename Field<P>::R R;
     typedef typename Field<PX>::R RX;
     const long long n5 = (long long)g.Vh * g.Ls;
@@ -991,12 +997,26 @@ inline int pick_ns(int Ls, size_t elem) {
     return ns;
 }
 
-template <typename K>
-unsigned grid_size(K kernel, int threads, size_t smem, int ntiles, int sms) {
+// resident blocks per SM of a kernel and block shape, asked of the runtime once
+// per process, device and shape (the query takes longer than a launch)
+inline int blocks_per_sm(const void* kernel, int threads, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::tuple<const void*, int, int, size_t>, int> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const auto key = std::make_tuple(kernel, dev, threads, smem);
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = known.find(key);
+    if (it != known.end()) return it->second;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     if (per_sm < 1) per_sm = 1;
-    long long cap = (long long)per_sm * sms;
+    return known[key] = per_sm;
+}
+
+template <typename K>
+unsigned grid_size(K kernel, int threads, size_t smem, int ntiles, int sms) {
+    long long cap = (long long)blocks_per_sm((const void*)kernel, threads, smem) * sms;
     if (cap > RED_MAX_BLOCKS) cap = RED_MAX_BLOCKS;
     return (unsigned)(ntiles < cap ? (ntiles > 0 ? ntiles : 1) : cap);
 }
@@ -1024,7 +1044,7 @@ void launch_with(K k, const eofa_ctx* ctx, const Geom& g, int NS, int spt, size_
     ep.aux2 = nullptr;
     ep.it = 0;
     ep.slot2 = 0;
-    k<<<grid, threads, smem, st>>>(g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
+    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
 }
 
 // direct kernel with a multi-output epilogue (MODE 1, 2) at NS sites per tile
@@ -1037,7 +1057,7 @@ void launch_epi(K k, const eofa_ctx* ctx, const Geom& g, int NS, size_t elem, bo
     const int ntiles = (g.Vh + NS - 1) / NS;
     if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     unsigned grid = grid_size(k, threads, smem, ntiles, ctx->sms);
-    k<<<grid, threads, smem, st>>>(g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
+    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
 }
 
 // Staged (bulk-copy) configurations are encoded as CFG_BULK | D << 8 | NS,
@@ -1291,7 +1311,7 @@ void launch_local5_t(const eofa_ctx* ctx, const Op5& op, const void* x, const vo
     auto k = local5_kernel<P, LS>;
     if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     unsigned grid = grid_size(k, threads, smem, ntiles, ctx->sms);
-    k<<<grid, threads, smem, st>>>(g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, NS);
+    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, NS);
     EOFA_LAUNCHED();
 }
 
@@ -1334,7 +1354,7 @@ void xp_update_prec(const eofa_ctx* ctx, const double* sc, int it, void* x, void
     long long nb = (n5 + 255) / 256;
     long long cap = (long long)ctx->sms * 8;
     unsigned grid = (unsigned)(nb < cap ? nb : cap);
-    xp_update_kernel<P, PX><<<grid, 256, 0, st>>>(g, sc, it, x, p, s);
+    launch_chained(nb <= cap, xp_update_kernel<P, PX>, grid, 256, 0, st, g, sc, it, x, p, s);
     EOFA_LAUNCHED();
 }
 

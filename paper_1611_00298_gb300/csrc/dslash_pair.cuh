@@ -601,6 +601,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 4)
     dslash_pair_kernel(Geom g, int par, const void* __restrict__ in, void* out, const void* __restrict__ gauge, PairOp op,
                        Op5 r1, PairOp op2, Op5 r2, const void* y, float a_out, float b_in, double* red, int slot, int NS,
                        ZBlocks zb, EpiPair ep) {
+    chain_wait();
     pair_body<P, DAG, LS, HASOP, MODE>(g, par, in, out, gauge, op, r1, op2, r2, y, a_out, b_in, red, slot, NS, zb,
                                               ep);
 }
@@ -640,9 +641,10 @@ inline bool pair_op_of(const Op5& op, int Ls, bool up, double factor, PairOp& o)
         o.c1[h] = (float)c1;
         o.k0[h] = (float)(c1 * mr + c2);
         o.k1[h] = (float)((c1 * mr + c2) * mr);
-        o.cor[h] = (float)(-op.mass / (1.0 + op.mass * std::pow(mr, Ls)));
+        o.cor[h] = (float)(-op.mass * op.nrm[h]);
         o.sig[h] = (float)(op.sigma[h] * f);
-        for (int i = 0; i < Ls / 2; i++) o.pw[h][i] = (float)std::pow(mr, 2 * i);
+        double p = 1.0;
+        for (int i = 0; i < Ls / 2; i++, p *= mr * mr) o.pw[h][i] = (float)p;
     }
     return true;
 }
@@ -684,10 +686,11 @@ void launch_pair(const eofa_ctx* ctx, int par, const PairArgs& a, const PairOp& 
     Geom g = ctx_geom(ctx);
     const PairShape s = pair_shape(g.Ls, HASOP);
     auto k = dslash_pair_kernel<P, DAG, LS, HASOP, MODE>;
-    const unsigned grid = grid_size(k, s.threads, s.smem, (g.Vh + s.NS - 1) / s.NS, ctx->sms);
-    k<<<grid, s.threads, s.smem, st>>>(g, par, a.in, a.out, ctx->gauge[P32], o, a.op ? *a.op : Op5(), o2,
-                                       a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
-                                       z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
+    const int ntiles = (g.Vh + s.NS - 1) / s.NS;
+    const unsigned grid = grid_size(k, s.threads, s.smem, ntiles, ctx->sms);
+    launch_chained((int)grid == ntiles, k, grid, s.threads, s.smem, st, g, par, a.in, a.out, (const void*)ctx->gauge[P32], o,
+                   a.op ? *a.op : Op5(), o2, a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
+                   z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
     EOFA_LAUNCHED();
 }
 
