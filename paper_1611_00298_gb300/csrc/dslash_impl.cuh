@@ -162,10 +162,21 @@ __device__ __forceinline__ void project(const cpx<R>* psi, cpx<R>* h) {
 __device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
 
-// u . h (three complex products) as two chains of multiply-adds, 12
+// c + u . h (three complex products) as two chains of multiply-adds, 12
 // instructions instead of the 16 of three products and two sums: the FP64
 // hop runs at the FP64 pipe's rate (1056 instructions a site and slice at
 // 24^3 x 64 x 24 in 20.9 ms), so its time is the instruction count.
+template <typename R>
+__device__ __forceinline__ cpx<R> row_dot_add(const cpx<R>* u, const cpx<R>* h, cpx<R> c) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        c.re = fma_r(u[k].re, h[k].re, c.re);
+        c.im = fma_r(u[k].re, h[k].im, c.im);
+        c.re = fma_r(-u[k].im, h[k].im, c.re);
+        c.im = fma_r(u[k].im, h[k].re, c.im);
+    }
+    return c;
+}
 template <typename R>
 __device__ __forceinline__ cpx<R> row_dot(const cpx<R>* u, const cpx<R>* h) {
     R re = u[0].re * h[0].re, im = u[0].re * h[0].im;
@@ -203,6 +214,39 @@ __device__ __forceinline__ void mac_row(const cpx<R>* u, int a, const cpx<R>* h,
     acc[9 + a] = SG > 0 ? acc[9 + a] + l1 : acc[9 + a] - l1;
 }
 
+// Both directions of MU at once (one slice): with w_f, w_b the rows of the
+// forward and the backward link the upper spins take t = w_f + w_b, whose
+// second half continues the chain of the first, and the lower ones
+// A^+ (w_b - w_f) = A^+ (t - 2 w_f) (SG < 0; else its negative): 30
+// instructions a row and spin instead of 32, 792 a site and slice instead of
+// 840.  16^3 x 32 x 12 FP64 hop: 1.61 ms with separate products and sums,
+// 1.25 with chains, 1.16 with chains over both directions.
+template <int MU, int SG, bool FIRST, typename R>
+__device__ __forceinline__ void mac_rows(const cpx<R>* uf, const cpx<R>* ub, int a, const cpx<R>* hf, const cpx<R>* hb,
+                                         cpx<R>* acc) {
+    cpx<R> t[2], e[2];
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const cpx<R> w = row_dot(uf, hf + 3 * q);
+        t[q] = row_dot_add(ub, hb + 3 * q, w);
+        e[q] = mk(fma_r(R(-2), w.re, t[q].re), fma_r(R(-2), w.im, t[q].im));
+    }
+    cpx<R> l0, l1;
+    if (MU == 0) { l0 = itimes(e[1]); l1 = itimes(e[0]); }
+    else if (MU == 1) { l0 = e[1]; l1 = mk(-e[0].re, -e[0].im); }
+    else if (MU == 2) { l0 = itimes(e[0]); l1 = mitimes(e[1]); }
+    else { l0 = e[0]; l1 = e[1]; }
+    acc[a] = FIRST ? t[0] : acc[a] + t[0];
+    acc[3 + a] = FIRST ? t[1] : acc[3 + a] + t[1];
+    if (SG < 0) {
+        acc[6 + a] = FIRST ? l0 : acc[6 + a] + l0;
+        acc[9 + a] = FIRST ? l1 : acc[9 + a] + l1;
+    } else {
+        acc[6 + a] = FIRST ? mk(-l0.re, -l0.im) : acc[6 + a] - l0;
+        acc[9 + a] = FIRST ? mk(-l1.re, -l1.im) : acc[9 + a] - l1;
+    }
+}
+
 // One direction pair for SPT slices s[0..SPT) of site j: the neighbour index
 // and every link row are loaded once and used for all SPT slices.
 template <int P, int DAG, int MU, int SPT>
@@ -210,6 +254,26 @@ __device__ __forceinline__ void hop_mu(const Geom& g, int par, int j, const int*
                                        long long n5, const void* in, const void* gauge,
                                        cpx<typename Field<P>::R> (*acc)[12]) {
     typedef typename Field<P>::R R;
+    if constexpr (P == P64 && SPT == 1) {
+        cpx<R> hf[6], hb[6];
+        {
+            cpx<R> psi[12];
+            Field<P>::load(in, ent[2 * MU], sv[0], Ls, n5, psi);
+            project<MU, DAG ? 1 : -1>(psi, hf);
+            Field<P>::load(in, ent[2 * MU + 1], sv[0], Ls, n5, psi);
+            project<MU, DAG ? -1 : 1>(psi, hb);
+        }
+        const long long lf = (long long)((par * 4 + MU) * g.Vh + j);
+        const long long lb = (long long)(((1 - par) * 4 + MU) * g.Vh + ent[2 * MU + 1]);
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            cpx<R> uf[3], ub[3];
+            link_row<R>(gauge, lf, a, false, uf);
+            link_row<R>(gauge, lb, a, true, ub);
+            mac_rows<MU, DAG ? 1 : -1, MU == 0>(uf, ub, a, hf, hb, acc[0]);
+        }
+        return;
+    }
 #pragma unroll
     for (int dirn = 0; dirn < 2; dirn++) {
         const int e = EOFA_HOP_PREFETCH ? ent[2 * MU + dirn]
@@ -1217,8 +1281,10 @@ int tuned_cfg(K1 k1, KB kb, KP2 kp2, KP3 kp3, const eofa_ctx* ctx, const Geom& g
     return best;
 }
 
-// Two slices per thread (SPT = 2) was measured slower than one in every tile
-// shape at 24^3 x 64 x 24 (0.79 vs 0.69 ms, FP32 hop), so only SPT = 1 is built.
+// FP32 and FP16 fields with an even Ls take the two-slice kernels
+// (dslash_pair.cuh) before they get here; this kernel's own SPT = 2 form
+// (slices Ls / 2 apart) was slower than SPT = 1 in every tile shape at 24^3 x
+// 64 x 24 (0.79 vs 0.69 ms, FP32 hop) and is not built.
 template <int P, int DAG, int LS>
 void launch_dslash_t(const eofa_ctx* ctx, int par, const void* in, void* out, const Op5& op, const void* y,
                      double a_out, double b_in, double* red, int slot, cudaStream_t st) {
