@@ -107,28 +107,6 @@ Op5 op_base() {
 
 }  // namespace
 
-Op5 op_finalize(Op5 op, int Ls) {
-    if (op.fin == Ls) return op;
-    op.fin = Ls;
-    for (int h = 0; h < 2; h++) {
-        if (op.inv[h]) {
-            op.mr[h] = -op.q1[h] / op.p1[h];
-            op.invp[h] = 1.0 / op.p1[h];
-            op.nrm[h] = 1.0 / (1.0 + op.mass * std::pow(op.mr[h], Ls));
-            op.invN[h] = 1.0 / (op.p1[h] * (1.0 + op.mass * std::pow(op.mr[h], Ls)));
-        } else {
-            op.mr[h] = op.invp[h] = op.invN[h] = op.nrm[h] = 0.0;
-        }
-        op.lead[h] = op.ratio[h] = op.sigl[h] = 0.0;
-        if (op.inv[h] && (!op.fwd[h] || (op.p2[h] != 0.0 && op.dir2[h] == op.dir1[h]))) {
-            op.lead[h] = (op.fwd[h] ? op.p2[h] : 1.0) * op.invp[h];
-            op.ratio[h] = op.fwd[h] ? op.q2[h] / op.p2[h] : 0.0;
-            op.sigl[h] = op.fwd[h] ? op.sigma[h] / op.p2[h] : op.sigma[h];
-        }
-    }
-    return op;
-}
-
 Coeffs make_coeffs(double alpha, double M5, double m) {
     Coeffs k;
     double c = 0.5 * alpha, d = 0.5;

@@ -131,10 +131,6 @@ void Solve::setup(eofa_ctx* c, const eofa_solve_params& prm, const double* b_dev
         G = op_G(ctx, S, base + 4, st);
     }
 
-    Gi = op_finalize(Gi, ctx->Ls);  // once a solve instead of at every launch
-    GiT = op_finalize(GiT, ctx->Ls);
-    G = op_finalize(G, ctx->Ls);
-
     const size_t f64 = field_bytes(P64, ctx->Vh, ctx->Ls);
     const long long n5full = (long long)ctx->V * ctx->Ls * 12;
     f_e = ctx_buffer(ctx, "sv_fe" + tag, f64);
