@@ -1108,7 +1108,8 @@ void launch_with(K k, const eofa_ctx* ctx, const Geom& g, int NS, int spt, size_
     ep.aux2 = nullptr;
     ep.it = 0;
     ep.slot2 = 0;
-    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
+    launch_chained(chain_pays(elem == sizeof(cpx<double>) ? CHAIN_F64 : CHAIN_ONE, grid, (int)grid == ntiles, ctx->sms), k,
+                   grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
 }
 
 // direct kernel with a multi-output epilogue (MODE 1, 2) at NS sites per tile
@@ -1121,7 +1122,8 @@ void launch_epi(K k, const eofa_ctx* ctx, const Geom& g, int NS, size_t elem, bo
     const int ntiles = (g.Vh + NS - 1) / NS;
     if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     unsigned grid = grid_size(k, threads, smem, ntiles, ctx->sms);
-    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
+    launch_chained(chain_pays(elem == sizeof(cpx<double>) ? CHAIN_F64 : CHAIN_ONE, grid, (int)grid == ntiles, ctx->sms), k,
+                   grid, threads, smem, st, g, par, in, out, gauge, op, y, a_out, b_in, red, slot, NS, ep);
 }
 
 // Staged (bulk-copy) configurations are encoded as CFG_BULK | D << 8 | NS,
@@ -1377,7 +1379,8 @@ void launch_local5_t(const eofa_ctx* ctx, const Op5& op, const void* x, const vo
     auto k = local5_kernel<P, LS>;
     if (smem > 40 * 1024) EOFA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     unsigned grid = grid_size(k, threads, smem, ntiles, ctx->sms);
-    launch_chained((int)grid == ntiles, k, grid, threads, smem, st, g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, NS);
+    launch_chained(chain_pays(P == P64 ? CHAIN_F64 : CHAIN_ONE, grid, (int)grid == ntiles, ctx->sms), k, grid, threads, smem, st,
+                   g, op, x, z, c0, sc, it, use_alpha, xw, out, a_out, y, b_in, red, slot, NS);
     EOFA_LAUNCHED();
 }
 
@@ -1420,7 +1423,8 @@ void xp_update_prec(const eofa_ctx* ctx, const double* sc, int it, void* x, void
     long long nb = (n5 + 255) / 256;
     long long cap = (long long)ctx->sms * 8;
     unsigned grid = (unsigned)(nb < cap ? nb : cap);
-    launch_chained(nb <= cap, xp_update_kernel<P, PX>, grid, 256, 0, st, g, sc, it, x, p, s);
+    launch_chained(chain_pays(P == P64 ? CHAIN_F64 : CHAIN_STREAM, grid, nb <= cap, ctx->sms), xp_update_kernel<P, PX>, grid, 256, 0,
+                   st, g, sc, it, x, p, s);
     EOFA_LAUNCHED();
 }
 

@@ -690,8 +690,8 @@ void launch_pair(const eofa_ctx* ctx, int par, const PairArgs& a, const PairOp& 
     auto k = dslash_pair_kernel<P, DAG, LS, HASOP, MODE>;
     const int ntiles = (g.Vh + s.NS - 1) / s.NS;
     const unsigned grid = grid_size(k, s.threads, s.smem, ntiles, ctx->sms);
-    launch_chained((int)grid == ntiles, k, grid, s.threads, s.smem, st, g, par, a.in, a.out, (const void*)ctx->gauge[P32], o,
-                   a.op ? *a.op : Op5(), o2, a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
+    launch_chained(chain_pays(CHAIN_PAIR, grid, (int)grid == ntiles, ctx->sms), k, grid, s.threads, s.smem, st, g, par, a.in,
+                   a.out, (const void*)ctx->gauge[P32], o, a.op ? *a.op : Op5(), o2, a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
                    z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
     EOFA_LAUNCHED();
 }

@@ -9,6 +9,7 @@
 #include <map>
 
 #include "../../include/eofa.h"
+#include "chain_rule.h"
 #include "op5.h"
 
 // ------------------------------------------------------------------ complex
@@ -137,9 +138,7 @@ struct eofa_error {
 // (programmatic stream serialization); every kernel launched so starts with
 // chain_wait(), which returns when the kernels before it have finished and
 // their writes are visible, so the order of all reads and writes is that of
-// plain launches.  chain: false for grids of more than one wave, where the gap
-// between kernels does not show (16^4 x 16: FP32 iteration 0.282 ms either way,
-// FP16 0.252 plain and 0.279 chained; 4^4 x 8 FP32 48 us plain, 41 chained).
+// plain launches.  chain: whether the overlap pays (chain_pays, chain_rule.h).
 // Inside a stream capture the launch is a plain one.
 template <typename... KP, typename... A>
 void launch_chained(bool chain, void (*k)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
