@@ -37,12 +37,19 @@ __global__ void pack_kernel(Geom g, int V, const double* __restrict__ canon, voi
 
 // A canonical slice holds a site's 12 components together (192 bytes), a device
 // field a component's Ls slices.  Unpacking with one thread per (site, slice)
-// writes through the canonical side with a whole slice between the lanes
-// (16^3 x 32 x 12 FP64: 212 us for 604 MB), so a block takes NJ pairs of
-// lexically neighbouring sites (one of each parity) with all their slices
-// through shared memory and writes runs of whole sectors: 154 us.  Packing keeps
-// the direct form: there the strided side is read, L1 collects the sectors
-// (109 us; through shared memory 129).
+// writes through the canonical side with a whole slice between the lanes, so a
+// block takes NJ pairs of lexically neighbouring sites (one of each parity) with
+// all their slices through shared memory and writes runs of whole sectors.  A
+// thread's site and component are worked out once and kept for all its slices:
+// with the six divisions of the index in every element the kernel issued more
+// than it wrote (6 x 10 x 14 x 18 x 16, us, one thread a site and slice / divisions
+// an element / this form: FP64 20.8 / 22.6 / 14.4, FP16 20.5 / 26.7 / 15.5, with the
+// output in L2; 43 / 33 / 25 and 43 / 31 / 21 with it in memory; 16^4 x 16: 156 /
+// 104 / 74 and 167 / 94 / 59).  10 pairs are at most 240 sites x components for
+// the 256 threads; for Ls < 5, where each has few slices, 16 pairs in two rounds
+// are faster (16^3 x 32 x 4 FP64 45 us instead of 54).
+// Packing keeps the direct form: there the strided side is read, L1 collects the
+// sectors (16^3 x 32 x 12 109 us; through shared memory 129).
 struct Block5 {
     int NJ, LsP;  // site pairs a block, stride of a component's slices (odd: conflict-free)
     int bytes;
@@ -52,25 +59,11 @@ inline Block5 block5(int Ls) {
     b.LsP = Ls | 1;
     const int per = 2 * 12 * b.LsP * 16;
     b.NJ = 40960 / per;
+    const int cap = Ls < 5 ? 16 : 10;
+    if (b.NJ > cap) b.NJ = cap;
     if (b.NJ < 1) b.NJ = 1;
-    if (b.NJ > 16) b.NJ = 16;
     b.bytes = b.NJ * per;
     return b;
-}
-
-// component e of slice s of the block's site k (0 .. 2 NJ - 1) on the canonical side, and where shared memory has it
-struct Canon {
-    int s, k, e, p;
-};
-__device__ __forceinline__ Canon canon_of(const Geom& g, int j0, int nk, int idx) {
-    Canon c;
-    c.e = idx % 12;
-    const int r = idx / 12;
-    c.k = r % nk;
-    c.s = r / nk;
-    const int i = 2 * j0 + c.k, x = i % g.X, rest = i / g.X;
-    c.p = (x + rest % g.Y + (rest / g.Y) % g.Z + rest / (g.Y * g.Z)) & 1;
-    return c;
 }
 
 template <int P>
@@ -89,10 +82,15 @@ __global__ void __launch_bounds__(256) unpack_kernel(Geom g, int V, const void* 
             sm[((p * b.NJ + jj) * 12 + c) * b.LsP + s] = make_double2((double)v[c].re, (double)v[c].im);
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nk * 12 * Ls; idx += blockDim.x) {
-        const Canon c = canon_of(g, j0, nk, idx);
-        __stcs((double2*)canon + ((long long)c.s * V + 2 * j0 + c.k) * 12 + c.e,
-               sm[((c.p * b.NJ + (c.k >> 1)) * 12 + c.e) * b.LsP + c.s]);
+    // a thread writes one component e of one site k (0 .. 2 NJ - 1) for every G-th slice
+    const int np = nk * 12, G = max(1, 256 / np);
+    for (int q = threadIdx.x; q < G * np; q += 256) {
+        const int pos = q % np, k = pos / 12, e = pos - 12 * k;
+        const int i = 2 * j0 + k, x = i % g.X, rest = i / g.X;
+        const int p = (x + rest % g.Y + (rest / g.Y) % g.Z + rest / (g.Y * g.Z)) & 1;
+        const double2* src = sm + ((p * b.NJ + (k >> 1)) * 12 + e) * b.LsP;
+        double2* dst = (double2*)canon + (long long)i * 12 + e;
+        for (int s = q / np; s < Ls; s += G) __stcs(dst + (long long)s * V * 12, src[s]);
     }
 }
 
