@@ -41,6 +41,7 @@
 #pragma once
 #include "dslash_impl.cuh"
 #include "mrhs.h"
+#include "pair_op.h"
 
 #include <algorithm>
 #include <climits>
@@ -300,18 +301,9 @@ __device__ __forceinline__ void hop_pair(const Geom& g, int par, int j, const in
 
 // ---------------------------------------------------------------- 5D-local block on pairs
 
-// B in the form v_s = x_s + mr v_{s-1}, out = c1 v_s + c2 v_{s-1} + w (sig vv . v),
-// mirrored in s for the chirality whose shift runs the other way.  On a pair
-// (x_0 first in its direction, k the carry):
-//   out_0 = c1 x_0 + k0 k,  out_1 = c1 x_1 + k0 x_0 + k1 k.
-struct PairOp {
-    float mr[2], m2[2], c1[2], k0[2], k1[2], cor[2], sig[2];
-    float pw[2][EOFA_MAX_LS / 2];  // mr^(2 i)
-};
-
 struct ColumnPlan {
     int lhp;              // stride of a column's carries (odd: conflict-free)
-    int carry, dot, sum;  // offsets in 8-byte units: carries, rank-one partial sums, rank-one sums
+    int carry, dot, sum;  // offsets in 8-byte units: carries, rank-one partial sums (one chirality's: pair_op_of), rank-one sums
     int bytes;
 };
 inline __host__ __device__ ColumnPlan column_plan(int NS, int Ls) {
@@ -631,26 +623,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, 4)
 
 // ---------------------------------------------------------------- launch
 
-// factor B as pair_op applies it; false for forms that it does not take.
-// up: direction of the upper chirality that the kernel is built for.
-inline bool pair_op_of(const Op5& op, int Ls, bool up, double factor, PairOp& o) {
-    for (int h = 0; h < 2; h++) {
-        if (!op.inv[h] || (op.fwd[h] && op.dir2[h] != op.dir1[h]) || (op.dir1[h] == 0) != (h == 0 ? up : !up)) return false;
-        const double mr = op.mr[h], f = factor * op.invp[h];
-        const double c1 = f * (op.fwd[h] ? op.p2[h] : 1.0), c2 = f * (op.fwd[h] ? op.q2[h] : 0.0);
-        o.mr[h] = (float)mr;
-        o.m2[h] = (float)(mr * mr);
-        o.c1[h] = (float)c1;
-        o.k0[h] = (float)(c1 * mr + c2);
-        o.k1[h] = (float)((c1 * mr + c2) * mr);
-        o.cor[h] = (float)(-op.mass * op.nrm[h]);
-        o.sig[h] = (float)(op.sigma[h] * f);
-        double p = 1.0;
-        for (int i = 0; i < Ls / 2; i++, p *= mr * mr) o.pw[h][i] = (float)p;
-    }
-    return true;
-}
-
 // A neighbour slab is fetched for t + 1 and used again for t and t - 1: three
 // slabs and the output have to stay in the L2 of a die (half of 126 MB, both
 // dies read most lines).  Slabs of up to 10 MB do; larger time slices are swept
@@ -691,8 +663,8 @@ void launch_pair(const eofa_ctx* ctx, int par, const PairArgs& a, const PairOp& 
     const int ntiles = (g.Vh + s.NS - 1) / s.NS;
     const unsigned grid = grid_size(k, s.threads, s.smem, ntiles, ctx->sms);
     launch_chained(chain_pays(CHAIN_PAIR, grid, (int)grid == ntiles, ctx->sms), k, grid, s.threads, s.smem, st, g, par, a.in,
-                   a.out, (const void*)ctx->gauge[P32], o, a.op ? *a.op : Op5(), o2, a.op2 ? *a.op2 : Op5(), a.y, (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS,
-                   z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
+                   a.out, (const void*)ctx->gauge[P32], o, a.op ? *a.op : Op5(), o2, a.op2 ? *a.op2 : Op5(), a.y,
+                   (float)a.a_out, (float)a.b_in, a.red, a.slot, s.NS, z_blocks(g, s.NS, P == P16 ? 52 : 96), e);
     EOFA_LAUNCHED();
 }
 
