@@ -73,10 +73,13 @@ struct Geom {
 // Kernel launch accounting and optional per-kernel CUDA-event timing.
 struct Prof {
     bool on = false;
-    int used = 0;
+    long long used = 0, taken = 0;  // launches since the start, and those of them whose pairs have been read
     std::vector<cudaEvent_t> ev;  // pairs (start, stop)
     std::vector<int> kind;        // 0..2 hop per precision, 3..5 op5 per precision
     std::vector<double> bytes;    // algorithmic bytes of each launch
+    // totals of the launches whose pairs have been read, per kind
+    long long launches[6] = {};
+    double ms[6] = {}, sum_bytes[6] = {};
 };
 // ------------------------------------------------------------------ context
 
