@@ -708,12 +708,22 @@ def main():
     return 0
 
 
-def kernel_version():
-    """Hash of the dslash kernel sources, to invalidate stored ncu traffic when they change."""
+def kernel_version(csrc=os.path.join(ROOT, "paper_1611_00298_gb300", "csrc")):
+    """Hash of the FP32 and FP16 dslash kernel sources and every source they include, to invalidate stored
+    ncu traffic when one changes."""
     import hashlib
+    import re
+    todo = ["dslash_pair_p32.cu", "dslash_pair_p16.cu", "dslash_p32.cu", "dslash_p16.cu"]
+    seen = {}
+    while todo:
+        f = todo.pop()
+        path = os.path.join(csrc, f)
+        if f not in seen and os.path.exists(path):
+            seen[f] = open(path, "rb").read()
+            todo += re.findall(r'#include "([^"/]+)"', seen[f].decode())
     h = hashlib.sha256()
-    for f in ("dslash_impl.cuh", "dslash_bulk.cuh", "dslash_pipe.cuh", "field.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_1611_00298_gb300", "csrc", f), "rb").read())
+    for f in sorted(seen):
+        h.update(f.encode() + b"\0" + seen[f])
     return h.hexdigest()[:16]
 
 
