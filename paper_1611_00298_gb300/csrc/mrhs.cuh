@@ -332,12 +332,17 @@ void mr_dslash_prec(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtr
 #define MR_CASE(L)                                                                                            \
     if (dag) mr_dslash_t<P, 1, L>(ctx, par, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st); \
     else mr_dslash_t<P, 0, L>(ctx, par, mode, a, ops, ops2, nr, hasop, a_out, b_in, slot, it, slot2, st);
-    switch (ctx->Ls) {
-        case 8: MR_CASE(8) break;
-        case 12: MR_CASE(12) break;
-        case 16: MR_CASE(16) break;
-        case 24: MR_CASE(24) break;
-        default: MR_CASE(0) break;
+    // (FP32 and FP16 systems with an even Ls run on the two-slice kernels: only odd Ls get here)
+    if constexpr (P != P64) {
+        MR_CASE(0)
+    } else {
+        switch (ctx->Ls) {
+            case 8: MR_CASE(8) break;
+            case 12: MR_CASE(12) break;
+            case 16: MR_CASE(16) break;
+            case 24: MR_CASE(24) break;
+            default: MR_CASE(0) break;
+        }
     }
 #undef MR_CASE
 }
