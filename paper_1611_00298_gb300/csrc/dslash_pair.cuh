@@ -734,6 +734,7 @@ void mr_pair_ls(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a
         launch_mr_pair<P, 0, LS, true, 0>(ctx, par, a, po, ops, po, ops2, nr, a_out, b_in, slot, it, slot2, st);
 }
 
+// (unrolled builds as for one system; eight systems on 8^4 x 24: 103 -> 97 ms in FP32, 100 -> 97 in FP16)
 template <int P>
 void mr_pair(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a, const void* pops, const Op5* ops,
              const Op5* ops2, int nr, double a_out, double b_in, int slot, int it, int slot2, cudaStream_t st) {
@@ -742,6 +743,7 @@ void mr_pair(const eofa_ctx* ctx, int par, int dag, int mode, const MRPtrs& a, c
         case 8: mr_pair_ls<P, 8>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
         case 12: mr_pair_ls<P, 12>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
         case 16: mr_pair_ls<P, 16>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
+        case 24: mr_pair_ls<P, 24>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
         default: mr_pair_ls<P, 0>(ctx, par, dag, mode, a, po, ops, ops2, nr, a_out, b_in, slot, it, slot2, st); break;
     }
 }
