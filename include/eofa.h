@@ -437,7 +437,8 @@ typedef struct {
 long long eofa_kernel_launches(void);
 /* Measured FP64 fused multiply-add rate of the current device in TFLOP/s
  * (2 flops per FMA; 8 independent chains per thread, best of 3 timed
- * launches): the ALU roofline of the FP64 hop.  Allocates 8 bytes. */
+ * launches), the scale for the FP64 hop; not an upper bound: kernels that mix
+ * FP64 with other instructions sustain some 5% more.  Allocates 8 bytes. */
 int eofa_probe_fp64_fma(double* tflops);
 int eofa_profile_start(eofa_ctx* ctx);
 int eofa_profile_stop(eofa_ctx* ctx, eofa_profile* out);

@@ -51,8 +51,10 @@ namespace {
 
 // ---------------------------------------------------------------- packed FP32 pairs
 // (re, im) of one complex number in a 64-bit register; the f32x2 instructions
-// do two FP32 multiply-adds each (used by the 5D-local recurrences; the same
-// form in the link products of the hop measured slower).
+// do two FP32 multiply-adds each (used by the 5D-local recurrences).  In the
+// link products of this kernel the form is slower, since a complex product
+// needs its halves swapped; with two slices in the halves (dslash_pair.cuh) it
+// needs no swaps and is the faster one.
 #ifndef EOFA_PACKED_F32
 #define EOFA_PACKED_F32 1
 #endif
@@ -220,7 +222,11 @@ __device__ __forceinline__ void mac_row(const cpx<R>* u, int a, const cpx<R>* h,
 // A^+ (w_b - w_f) = A^+ (t - 2 w_f) (SG < 0; else its negative): 30
 // instructions a row and spin instead of 32, 792 a site and slice instead of
 // 840.  16^3 x 32 x 12 FP64 hop: 1.61 ms with separate products and sums,
-// 1.25 with chains, 1.16 with chains over both directions.
+// 1.25 with chains, 1.16 with chains over both directions.  The longer chain
+// costs part of a last bit: error against 64-bit torch 2.42e-16 (Ls 12) and
+// 2.35e-16 (Ls 7) of G^-1 hop with separate products, 2.53e-16 and 2.57e-16 so;
+// t and e as sums of two separate chains gave 2.43e-16 and 2.47e-16 at 840
+// instructions (1.25 ms).
 template <int MU, int SG, bool FIRST, typename R>
 __device__ __forceinline__ void mac_rows(const cpx<R>* uf, const cpx<R>* ub, int a, const cpx<R>* hf, const cpx<R>* hb,
                                          cpx<R>* acc) {

@@ -47,6 +47,8 @@
 #include <climits>
 #include <cmath>
 
+// 96 / (Ls / 2) whole sites a block: all threads at work for Ls 2, 4, 6, 8, 12, 16, 24,
+// 32, 48 and 64, at worst 75 of 96 (Ls 50)
 #define PAIR_THREADS 96
 namespace dsl {
 namespace {
@@ -628,7 +630,9 @@ __global__ void __launch_bounds__(PAIR_THREADS, 4)
 // dies read most lines).  Slabs of up to 10 MB do; larger time slices are swept
 // in blocks of z.  24^3 x 64 x 24, hop: FP32, 15.9 MB a slice, 0.594 ms
 // unblocked, 0.574 in two blocks, 0.579 in three, 0.594 in six; FP16, 8.6 MB,
-// 0.588 ms unblocked, 0.599 in two.
+// 0.588 ms unblocked, 0.599 in two.  A block's slab has to hold whole tiles:
+// where no count of blocks divides it so (32^3 x Ls 16: tiles of 12 sites, slabs
+// of 16384; most Ls that are no divisor of 192) the sweep stays unblocked.
 inline ZBlocks z_blocks(const Geom& g, int NS, int spinor) {
     const long long slice = (long long)(g.X / 2) * g.Y * g.Z;
     ZBlocks z = {1, 0};

@@ -133,7 +133,7 @@ __device__ __forceinline__ void link_Y(const double2* chiL, const double2* chiR,
 //
 // Bound by the FP64 pipe: 24 additions for the half spinors, 72 multiply-adds
 // for the outer product and 4.5 additions of partial sums per link, slice and
-// chi (24^3 x 32 x 24: 8.5e9 of them, 16 ms at the measured 1.057 TFLOP/s).  A block works on one
+// chi (24^3 x 32 x 24: 8.5e9 of them, 13.6 ms at the nominal 1.25 TFLOP/s).  A block works on one
 // direction (the four blocks of a run of sites are neighbours in the grid and
 // share their spinors in L2): with the four directions in the lanes of a warp,
 // as before, every warp ran all four one after another, and with products

@@ -14,7 +14,8 @@
 //
 // Blocks without an inverse (D-tilde, M) are a two-point stencil in s: one
 // thread per (site, s) reads its slice and, through L1, the neighbouring one
-// of each chirality.  All others run as the launch of the CG's residual update
+// of each chirality.  All others, and a stencil that writes its own input (the
+// D-tilde^T passes of D_DWF^+), run as the launch of the CG's residual update
 // without its update (local5_kernel, dslash_impl.cuh): whole 4D sites staged in
 // shared memory, one thread per (site, component) column.
 //

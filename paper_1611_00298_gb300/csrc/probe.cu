@@ -1,7 +1,11 @@
 // Instrumentation: the FP64 fused multiply-add rate of the current GPU,
 // the ALU roofline of the FP64 hop (GB300 has a reduced FP64 rate and no
 // measured FP64 peak).  Every thread runs 8 independent dependency
-// chains of a = a * b + c, so the FP64 pipe, not latency, sets the time.
+// chains of a = a * b + c, so the FP64 pipe, not latency, sets the time (4, 8
+// and 16 chains and 4 to 64 warps an SM give the same rate).  The rate moves in
+// steps from box to box and run to run, 1.008 or 1.057 TFLOP/s at an SM clock of
+// 1995 MHz with no throttle reason set; kernels that mix FP64 with other
+// instructions sustain 1.10, so it is no upper bound for them (nominal: 1.25).
 #include "api_util.h"
 
 namespace {
